@@ -1,6 +1,6 @@
 """Build libftk.so (the C-ABI library of include/ftk.h) in-tree with nvcc.
 
-sm_103a only: -gencode arch=compute_103a,code=sm_103a. The two translation
+sm_103a only: -gencode arch=compute_103a,code=sm_103a. The translation
 units compile in parallel; the result lands next to this file and is loaded
 by the ctypes binding.
 """
@@ -15,7 +15,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libftk.so")
-SOURCES = ["ftk_api.cu", "ftk_kernels.cu", "ftk_hv.cu", "ftk_noalloc.cu", "ftk_sector.cu"]
+SOURCES = ["ftk_api.cu", "ftk_kernels.cu", "ftk_hv.cu", "ftk_gather.cu", "ftk_noalloc.cu", "ftk_sector.cu"]
 HEADERS = ["ftk_common.cuh", "ftk_kernels.h", "ftk_plan.h", "ftk_device.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-diag-suppress", "128"]

@@ -62,6 +62,7 @@ Layout make_layout(int n, int n_saved, int max_rhs, int prec) {
 struct Small {
     TpqState tpq;
     unsigned int counters[8];
+    unsigned int hv_counters[FTK_MAX_RHS];   // tickets of the products' reductions, per column
     double hv_dots[FTK_MAX_RHS * FTK_HV_DOTS];
     double upd_dots[FTK_MAX_RHS * FTK_UPD_DOTS];
     double op_dots[4];
@@ -74,6 +75,7 @@ struct Small {
 struct Plan {
     int tile_bits = 0, chunk_bits = 0, threads = 512, grid = 0;
     size_t smem = 0;
+    bool gather = false;             // one launch over the whole vector (ftk_gather.cu), no passes
     std::vector<PassDesc> passes;
 };
 
@@ -90,6 +92,7 @@ struct ftk_ctx {
     uint64_t dim = 0;
     double K = 0, J = 0, ell_min = 0;
     std::vector<Bond> bonds;
+    GatherDesc gd{};
     std::vector<double> pos;
     cudaStream_t stream = nullptr;
     bool own_stream = false;
@@ -176,6 +179,13 @@ bool plan_passes(ftk_ctx *ctx, int prec, int bc, int tile_bits, Plan &pl) {
 ftk_status get_plan(ftk_ctx *ctx, int prec, int B, Plan **out) {
     auto it = ctx->plans.find(prec * 64 + B);
     if (it != ctx->plans.end()) { *out = &it->second; return FTK_OK; }
+    if (ctx->tile_bits_req <= 0 && hv_use_gather(prec, ctx->n, B)) {
+        Plan pl;
+        pl.gather = true;
+        pl.tile_bits = ctx->n;
+        *out = &ctx->plans.emplace(prec * 64 + B, pl).first->second;
+        return FTK_OK;
+    }
     // default: all columns in one launch (at most hv_max_b), the largest tile;
     // the FP32 products of a relaxed double-float solve: one column per
     // launch (the largest tile, fewest passes)
@@ -205,6 +215,10 @@ ftk_status run_hv(ftk_ctx *ctx, int prec, int B, int epi, const void *in, void *
     Plan *pl = nullptr;
     ftk_status s = get_plan(ctx, prec, B, &pl);
     if (s != FTK_OK) return s;
+    if (pl->gather) {
+        LAUNCH(launch_hv_gather(prec, B, epi, in, out, ctx->gd, ea, ctx->stream));
+        return FTK_OK;
+    }
     const int np = (int)pl->passes.size();
     for (int p = 0; p < np; ++p) {
         const int e = (p == np - 1) ? epi : EPI_PLAIN;
@@ -355,7 +369,9 @@ ftk_status ftk_create(const ftk_lattice *lat, const ftk_bond *bonds, int32_t n_b
         return fail(nullptr, FTK_ECUDA, std::string("kernel attributes: ") + cudaGetErrorString(ka));
     }
     Plan *pl = nullptr;
-    if (get_plan(ctx, ctx->mprec, 1, &pl) != FTK_OK) {
+    PlanBond pb[2 * FTK_MAX_PASS_BONDS];
+    for (int q = 0; q < n_bonds; ++q) pb[q] = {bonds[q].i, bonds[q].j, bonds[q].gamma};
+    if (!gather_desc(n, pb, n_bonds, K, J, &ctx->gd) || get_plan(ctx, ctx->mprec, 1, &pl) != FTK_OK) {
         std::string m = ctx->err;
         ftk_destroy(ctx);
         return fail(nullptr, FTK_EINVAL, m);
@@ -629,14 +645,28 @@ static ftk_status cocg_iteration(ftk_ctx *ctx, int B, void *rcur, void *rprev, v
             ea.lowp_run = 0;
         }
         ea.df_lo = ua.lo_stride;
-        ea.fu_seed = ua.seed;
-        ea.fu_rcur = static_cast<float2 *>(rcur);
-        ea.fu_lam = ua.lam_split;
-        ea.fu_result = ua.result;
-        ftk_status s = run_hv(ctx, ctx->mprec, B, EPI_COCG, rprev, w, ea);
-        if (s) return s;
+        Plan *pl = nullptr;
+        ftk_status ps = get_plan(ctx, ctx->mprec, B, &pl);
+        if (ps) return ps;
+        if (pl->gather) {
+            // the gather reads its partners' finished residuals: the update
+            // is a launch of its own
+            UpdArgs u = ua;
+            u.mode = 1;
+            u.lowp = ea.lowp;
+            u.lowp_run = 0;
+            LAUNCH(launch_cocg_update(upd_kind(ctx), B, rcur, w, rprev, u, vec_grid(ctx, ctx->dim), ctx->stream));
+            if ((ps = run_hv(ctx, ctx->mprec, B, EPI_COCG, rprev, w, ea))) return ps;
+        } else {
+            ea.fu_seed = ua.seed;
+            ea.fu_rcur = static_cast<float2 *>(rcur);
+            ea.fu_lam = ua.lam_split;
+            ea.fu_result = ua.result;
+            if ((ps = run_hv(ctx, ctx->mprec, B, EPI_COCG, rprev, w, ea))) return ps;
+        }
         LAUNCH(launch_cocg_seed(sa, ctx->stream));
-        // the new r_k is the buffer rprev (written by the fused update), r_{k-1} is rcur
+        // the new r_k is the buffer rprev (written by the update), r_{k-1} is rcur
+        ftk_status s = FTK_OK;
         if ((s = after_seed(rprev, rcur))) return s;
         LAUNCH(launch_cocg_shift(sh, B, ctx->stream));
         return FTK_OK;
@@ -771,9 +801,10 @@ static ftk_status cocg_core(ftk_ctx *ctx, const CocgReq &rq, double *G_out, int3
     ua.lam_split = reinterpret_cast<float4 *>(wsp(ctx, ctx->L.lam_split));
     EpiArgs ea{};
     ea.partials = (double *)wsp(ctx, ctx->L.partials);
-    ea.counter = &d->counters[4];
+    ea.counter = d->hv_counters;
     ea.result = d->hv_dots;
     ea.all_done = &d->all_done;
+    ea.col_seed = d->seed;
     SeedArgs sa{};
     sa.n_rhs = B;
     sa.max_iter = rq.max_iter;
@@ -1433,7 +1464,7 @@ ftk_status ftk_plan_info(const ftk_ctx *cctx, int32_t *n_passes, int32_t *tile_b
     Plan *pl = nullptr;
     ftk_status s = get_plan(ctx, ctx->mprec, 1, &pl);
     if (s) return s;
-    if (n_passes) *n_passes = (int)pl->passes.size();
+    if (n_passes) *n_passes = pl->gather ? 1 : (int)pl->passes.size();
     if (tile_bits) *tile_bits = pl->tile_bits;
     return FTK_OK;
 }
@@ -1467,34 +1498,43 @@ ftk_status ftk_autotune(ftk_ctx *ctx, int32_t n_rhs, int32_t which, int32_t *til
     EpiArgs ea{};
     if (prec == 2) ea.df_lo = (long long)n_rhs * (long long)ctx->dim;
     ftk_status st = FTK_OK;
+    auto time_plan = [&](const Plan &pl) {
+        for (int rep = 0; rep < 4; ++rep) {
+            if (rep == 1 && cudaEventRecord(e0, ctx->stream) != cudaSuccess) st = FTK_ECUDA;
+            if (pl.gather && launch_hv_gather(prec, n_rhs, EPI_PLAIN, in, out, ctx->gd, ea, ctx->stream) != cudaSuccess)
+                st = FTK_ECUDA;
+            for (size_t p = 0; p < pl.passes.size() && st == FTK_OK; ++p)
+                if (launch_hv_pass(prec, n_rhs, EPI_PLAIN, in, out, pl.passes[p], ea, pl.grid, ctx->stream) !=
+                    cudaSuccess)
+                    st = FTK_ECUDA;
+        }
+        float ms = 0;
+        if (st == FTK_OK && (cudaEventRecord(e1, ctx->stream) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess ||
+                             cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess))
+            st = FTK_ECUDA;
+        const double us = 1e3 * ms / 3;
+        if (st == FTK_OK && us < best_us) { best_us = us; best = pl; }
+    };
     for (int bc = 1; bc <= std::min((int)n_rhs, hv_max_b(prec)) && st == FTK_OK; bc <<= 1) {
         const int tb_max = std::min(hv_max_tile_bits(prec, bc), ctx->n);
         for (int tb = std::max(5, tb_max - 2); tb <= tb_max && st == FTK_OK; ++tb) {
             Plan pl;
-            if (!plan_passes(ctx, prec, bc, tb, pl)) continue;
-            for (int rep = 0; rep < 4; ++rep) {
-                if (rep == 1 && cudaEventRecord(e0, ctx->stream) != cudaSuccess) st = FTK_ECUDA;
-                for (size_t p = 0; p < pl.passes.size() && st == FTK_OK; ++p)
-                    if (launch_hv_pass(prec, n_rhs, EPI_PLAIN, in, out, pl.passes[p], ea, pl.grid, ctx->stream) !=
-                        cudaSuccess)
-                        st = FTK_ECUDA;
-            }
-            float ms = 0;
-            if (st == FTK_OK && (cudaEventRecord(e1, ctx->stream) != cudaSuccess ||
-                                 cudaEventSynchronize(e1) != cudaSuccess ||
-                                 cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess))
-                st = FTK_ECUDA;
-            const double us = 1e3 * ms / 3;
-            if (st == FTK_OK && us < best_us) { best_us = us; best = pl; }
+            if (plan_passes(ctx, prec, bc, tb, pl)) time_plan(pl);
         }
+    }
+    if (st == FTK_OK && hv_use_gather(prec, ctx->n, n_rhs)) {
+        Plan pl;
+        pl.gather = true;
+        pl.tile_bits = ctx->n;
+        time_plan(pl);
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (st != FTK_OK) return fail(ctx, st, "ftk_autotune: CUDA error while timing");
-    if (best.passes.empty()) return fail(ctx, FTK_EINVAL, "ftk_autotune: no admissible plan");
+    if (best.passes.empty() && !best.gather) return fail(ctx, FTK_EINVAL, "ftk_autotune: no admissible plan");
     ctx->plans[prec * 64 + n_rhs] = best;
     if (tile_bits_out) *tile_bits_out = best.tile_bits;
-    if (cols_out) *cols_out = best.passes[0].cols;
+    if (cols_out) *cols_out = best.gather ? n_rhs : best.passes[0].cols;
     if (us_out) *us_out = best_us;
     return FTK_OK;
 }

@@ -3,6 +3,7 @@
 // reductions (fixed summation order, no floating-point atomics).
 #pragma once
 #include "ftk_common.cuh"
+#include "ftk_kernels.h"
 
 namespace ftk {
 
@@ -140,6 +141,92 @@ template <> struct Coef<float> {
     __device__ static __forceinline__ float dgv(const PassDesc &p, int c) { return p.dgv_f[c]; }
 };
 
+// acc += c p for a complex amplitude and a real coefficient: on sm_100 and
+// later, float pairs take one packed FMA (fma.rn.f32x2) for both components
+__device__ __forceinline__ void cfma(double c, const double2 &p, double2 &acc) {
+    acc.x = fma(c, p.x, acc.x);
+    acc.y = fma(c, p.y, acc.y);
+}
+__device__ __forceinline__ void cfma(float c, const float2 &p, float2 &acc) {
+    acc = __ffma2_rn(make_float2(c, c), p, acc);
+}
+__device__ __forceinline__ void cadd(const double2 &p, double2 &acc) { acc.x += p.x; acc.y += p.y; }
+__device__ __forceinline__ void cadd(const float2 &p, float2 &acc) { acc = __fadd2_rn(acc, p); }
+
+// ------------------------------------------------------ H.V epilogues
+// What the last launch of a product does with an amplitude v and its finished
+// product w = (H v): store, and the dots of the mTPQ step, the Taylor term or
+// the COCG iteration. i: element index (column offset included).
+template <typename R, int EPI>
+struct HvEpilogue {
+    typedef typename C2<R>::t cx;
+    R scale, ell, inv_n, tcoef;
+    __device__ explicit HvEpilogue(const EpiArgs &ea)
+        : scale(EPI == EPI_TPQ ? (R)(*ea.scale) : (R)1), ell((R)ea.ell), inv_n((R)ea.inv_n),
+          tcoef(EPI == EPI_TAYLOR ? (R)ea.tcoef : (R)0) {}
+    template <typename D>
+    __device__ __forceinline__ void apply(const EpiArgs &ea, size_t i, const cx &v, const cx &w, cx *out, D *dot) const {
+        if constexpr (EPI == EPI_PLAIN) {
+            *out = w;
+        } else if constexpr (EPI == EPI_TPQ) {
+            // psi' = s (l v - H v / N);  <v|Hv>, |psi'|^2
+            const R yr = scale * (ell * v.x - inv_n * w.x);
+            const R yi = scale * (ell * v.y - inv_n * w.y);
+            *out = mk<R>(yr, yi);
+            dot[0].fma2(v.x, w.x);
+            dot[0].fma2(v.y, w.y);
+            dot[1].fma2(yr, yr);
+            dot[1].fma2(yi, yi);
+        } else if constexpr (EPI == EPI_TAYLOR) {
+            // cTPQ Taylor term: t' = c (l v - H v / N), acc += t';
+            // <v|Hv> (the energy of v), |acc|^2
+            const R yr = tcoef * (ell * v.x - inv_n * w.x);
+            const R yi = tcoef * (ell * v.y - inv_n * w.y);
+            *out = mk<R>(yr, yi);
+            cx *ap = reinterpret_cast<cx *>(ea.taylor_acc) + i;
+            cx a = *ap;
+            a.x += yr;
+            a.y += yi;
+            *ap = a;
+            dot[0].fma2(v.x, w.x);
+            dot[0].fma2(v.y, w.y);
+            dot[1].fma2(a.x, a.x);
+            dot[1].fma2(a.y, a.y);
+        } else if constexpr (EPI == EPI_COCG) {
+            // W = H R;  mu = R^T W (bilinear)
+            *out = w;
+            dot[0].fma2(v.x, w.x);
+            dot[0].fma2(-v.y, w.y);
+            dot[1].fma2(v.x, w.y);
+            dot[1].fma2(v.y, w.x);
+        } else if constexpr (EPI == EPI_COCG_MIXED) {
+            // mixed mode: R = hi + lo, mu = R^T W with exact FMA two-products
+            // and two-sums (double-float, ~48 bits) on the FP32 pipe
+            *out = w;
+            const float2 lo = reinterpret_cast<const float2 *>(ea.lo)[i];
+            dot[0].fma_hl(v.x, lo.x, w.x);
+            dot[0].fma_hl(-v.y, -lo.y, w.y);
+            dot[1].fma_hl(v.x, lo.x, w.y);
+            dot[1].fma_hl(v.y, lo.y, w.x);
+        }
+    }
+};
+// mTPQ statistics of step k (Appendix A) from the reduced dots, by one thread:
+// u_k = s^2 <v|Hv>/N, q_k = ||psi'||, <H^2>_k = N^2 (q^2 - l^2 + 2 l u_k)
+__device__ __forceinline__ void tpq_statistics(const EpiArgs &ea, const double *res) {
+    TpqState *stt = ea.tpq;
+    const double s = stt->scale, n = stt->n_sites, l = stt->ell;
+    const double u = s * s * res[0] / n;
+    const double q2 = res[1];
+    const int k = stt->k;
+    ea.stat_u[k] = u;
+    ea.stat_logq[k] = stt->logQ;
+    ea.stat_h2[k] = n * n * (q2 - l * l + 2.0 * l * u);
+    stt->logQ += 0.5 * log(q2);
+    stt->scale = 1.0 / sqrt(q2);
+    stt->k = k + 1;
+}
+
 }  // namespace ftk
 
 // ------------------------------------------------------------ double-float
@@ -213,6 +300,37 @@ __device__ __forceinline__ void dfl_mac(dfl &acc, dfl a, dfl b) {
 }
 // Renormalised pair of an accumulator (two-sum: no ordering assumption).
 __device__ __forceinline__ dfl dfl_renorm(dfl a) { return dfl_two_sum(a.hi, a.lo); }
+
+// Multiply-accumulate of a bond's term in the double-float product.
+// The real and imaginary components take the same operations with the same
+// coefficient, so every step runs on float pairs (re, im) as one packed
+// f32x2 instruction (sm_100 and later). No step negates an operand: a - b is
+// formed as fma(b, -1, a) (the same rounding as the subtraction) and the
+// product's error term from the negated coefficient -c_hi, so each complex
+// term costs 12 packed instructions. h, l: the (re, im) hi and lo parts of
+// the accumulator.
+__device__ __forceinline__ float2 m1x2() { return make_float2(-1.f, -1.f); }
+__device__ __forceinline__ float2 fsub2(float2 a, float2 b) { return __ffma2_rn(b, m1x2(), a); }   // a - b
+// acc += c p, c = ch + cl, p = ph + pl; nch = -ch, ncl = -cl:
+//   p_hh = ch ph;  en = -(ch ph - p_hh) - ch pl - cl ph  (exact first step)
+//   t = h + p_hh, Knuth two-sum error into l together with -en
+__device__ __forceinline__ void df_acc2(float2 &h, float2 &l, float2 ch, float2 nch, float2 ncl, float2 ph, float2 pl) {
+    const float2 p = __fmul2_rn(ch, ph);
+    float2 en = __ffma2_rn(nch, ph, p);
+    en = __ffma2_rn(nch, pl, en);
+    en = __ffma2_rn(ncl, ph, en);
+    const float2 t = __fadd2_rn(h, p);
+    const float2 bb = fsub2(t, h);
+    const float2 s = __fadd2_rn(fsub2(h, fsub2(t, bb)), fsub2(p, bb));
+    l = __fadd2_rn(l, fsub2(s, en));
+    h = t;
+}
+__device__ __forceinline__ void df_add_to2(float2 &h, float2 &l, float2 ph, float2 pl) {
+    const float2 t = __fadd2_rn(h, ph);
+    const float2 bb = fsub2(t, h);
+    l = __fadd2_rn(l, __fadd2_rn(__fadd2_rn(fsub2(h, fsub2(t, bb)), fsub2(ph, bb)), pl));
+    h = t;
+}
 
 // Three-term COCG residual (Sec. IV): with w_k = H r_k,
 // r_{k+1} = r_k + c_k (r_k - r_{k-1}) - alpha_k (z_s r_k - w_k)

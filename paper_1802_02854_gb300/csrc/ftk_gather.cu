@@ -1,0 +1,238 @@
+// The matrix-free H.V of vectors that sit in the L2 cache, in one launch: one
+// thread per amplitude reads its partners x ^ m of all bonds straight from
+// global memory.
+//
+// Why beside the tiled passes of ftk_hv.cu: a tile of 2^12 amplitudes is the
+// unit of work there, so a small vector occupies few SMs (12 sites: one tile,
+// hence one SM, and 36 us of its FP64 pipe; 16 sites: 16 SMs and two
+// launches), while here 2^n threads spread over all of them. The price is one
+// 16-byte L2 read per bond and amplitude instead of a shared-memory one, so
+// the tiles win again once the reads of a launch cost more than the passes'
+// launches and empty SMs (hv_use_gather, with both sides measured).
+#include "ftk_common.cuh"
+#include "ftk_device.cuh"
+#include "ftk_kernels.h"
+#include "ftk_plan.h"
+
+#include <algorithm>
+#include <type_traits>
+
+namespace ftk {
+
+// partners in flight per thread: the loads of a chunk are independent, and
+// their latency (not their bandwidth) is what a small launch waits for
+constexpr int kGatherChunk = 6;
+
+// One column's vector in each arithmetic: load an amplitude, add c times a
+// partner's, and the finished value.
+template <int PREC> struct GatherVec;
+template <> struct GatherVec<0> {
+    typedef double2 amp;
+    typedef double coef;
+    double2 s = {0.0, 0.0};
+    __device__ static amp load(const void *p, size_t i, long long) { return static_cast<const double2 *>(p)[i]; }
+    __device__ static coef c(const GatherDesc &g, int q, bool anti) { return anti ? g.anti[q] : g.par[q]; }
+    __device__ void add(coef c, const amp &a) { s.x = fma(c, a.x, s.x); s.y = fma(c, a.y, s.y); }
+    __device__ void diag(const GatherDesc &g, int c0, int c1, const amp &a) {
+        add((double)c0 * g.dgv[0] + (double)c1 * g.dgv[1], a);
+    }
+};
+template <> struct GatherVec<1> {
+    typedef float2 amp;
+    typedef float coef;
+    float2 s = {0.f, 0.f};
+    __device__ static amp load(const void *p, size_t i, long long) { return static_cast<const float2 *>(p)[i]; }
+    __device__ static coef c(const GatherDesc &g, int q, bool anti) { return anti ? g.anti_f[q] : g.par_f[q]; }
+    __device__ void add(coef c, const amp &a) { s = __ffma2_rn(make_float2(c, c), a, s); }
+    __device__ void diag(const GatherDesc &g, int c0, int c1, const amp &a) {
+        add((float)c0 * g.dgv_f[0] + (float)c1 * g.dgv_f[1], a);
+    }
+};
+template <> struct GatherVec<2> {
+    typedef float4 amp;    // (hi.re, hi.im, lo.re, lo.im)
+    typedef float2 coef;   // (hi, lo)
+    float2 h = {0.f, 0.f}, l = {0.f, 0.f};
+    __device__ static amp load(const void *p, size_t i, long long lo) {
+        const float2 *q = static_cast<const float2 *>(p) + i;
+        const float2 a = q[0], b = q[lo];
+        return make_float4(a.x, a.y, b.x, b.y);
+    }
+    __device__ static coef c(const GatherDesc &g, int q, bool anti) {
+        return anti ? make_float2(g.anti_f[q], g.anti_lo[q]) : make_float2(g.par_f[q], g.par_lo[q]);
+    }
+    __device__ void add(coef c, const amp &a) {
+        df_acc2(h, l, make_float2(c.x, c.x), make_float2(-c.x, -c.x), make_float2(-c.y, -c.y), make_float2(a.x, a.y),
+                make_float2(a.z, a.w));
+    }
+    __device__ void diag(const GatherDesc &g, int c0, int c1, const amp &a) {
+        const dfl d = dfl_add(dfl_mul({(float)c0, 0.f}, {g.dgv_f[0], g.dgv_lo[0]}),
+                              dfl_mul({(float)c1, 0.f}, {g.dgv_f[1], g.dgv_lo[1]}));
+        add(make_float2(d.hi, d.lo), a);
+    }
+    // the renormalised pair
+    __device__ amp value() const {
+        const float2 hh = __fadd2_rn(h, l);
+        const float2 ll = fsub2(l, fsub2(hh, h));
+        return make_float4(hh.x, hh.y, ll.x, ll.y);
+    }
+};
+
+// Grid (blocks, columns); element (x, j) at j 2^n + x. Reductions: per-block
+// partials of the column, summed in a fixed order by its last block.
+template <int PREC, int EPI>
+__global__ void __launch_bounds__(128) hv_gather_kernel(const void *__restrict__ in, void *out,
+                                                        const __grid_constant__ GatherDesc gd,
+                                                        const __grid_constant__ EpiArgs ea) {
+    typedef GatherVec<PREC> V;
+    typedef typename std::conditional<PREC == 0, double, float>::type R;
+    constexpr int ND = EPI == EPI_PLAIN ? 1 : 2;
+    __shared__ double red[(128 / 32) * ND];
+    const int j = blockIdx.y;
+    if (ea.all_done && *ea.all_done) return;
+    if (ea.lowp && *ea.lowp != ea.lowp_run) return;
+    if (ea.col_seed && ea.col_seed[j].done != 0) return;   // finished column: no work
+    const uint32_t dim = 1u << gd.n_sites;
+    const size_t base = (size_t)j * dim;
+    Acc<R> dot[ND];
+    for (uint32_t x = blockIdx.x * blockDim.x + threadIdx.x; x < dim; x += gridDim.x * blockDim.x) {
+        V acc;
+        int anti[3] = {0, 0, 0};
+#pragma unroll
+        for (int g = 0; g < 3; ++g) {
+            for (int b = gd.off[g]; b < gd.off[g + 1]; b += kGatherChunk) {
+                typename V::amp p[kGatherChunk];
+#pragma unroll
+                for (int u = 0; u < kGatherChunk; ++u)
+                    if (b + u < gd.off[g + 1]) p[u] = V::load(in, base + (x ^ gd.mask[b + u]), ea.df_lo);
+#pragma unroll
+                for (int u = 0; u < kGatherChunk; ++u)
+                    if (b + u < gd.off[g + 1]) {
+                        const int odd = __popc(x & gd.mask[b + u]) & 1;
+                        anti[g] += odd;
+                        acc.add(V::c(gd, g, odd != 0), p[u]);
+                    }
+            }
+        }
+        // diagonal: (parallel - antiparallel) bonds of the two classes
+        const int c0 = gd.off[2] - 2 * (anti[0] + anti[1]);
+        const int c1 = gd.off[3] - gd.off[2] - 2 * anti[2];
+        const typename V::amp v = V::load(in, base + x, ea.df_lo);
+        acc.diag(gd, c0, c1, v);
+        if constexpr (PREC == 2) {
+            const float4 w = acc.value();
+            float2 *o = static_cast<float2 *>(out) + base + x;
+            o[0] = make_float2(w.x, w.y);
+            o[ea.df_lo] = make_float2(w.z, w.w);
+            if constexpr (EPI == EPI_COCG) {   // mu = r^T w (bilinear) from hi + lo
+                dot[0].fma_pair(v.x, v.z, w.x, w.z);
+                dot[0].fma_pair(-v.y, -v.w, w.y, w.w);
+                dot[1].fma_pair(v.x, v.z, w.y, w.w);
+                dot[1].fma_pair(v.y, v.w, w.x, w.z);
+            }
+        } else {
+            typedef typename C2<R>::t cx;
+            cx *o = static_cast<cx *>(out) + base + x;
+            HvEpilogue<R, EPI>(ea).apply(ea, base + x, v, acc.s, o, dot);
+        }
+    }
+    if constexpr (EPI != EPI_PLAIN) {
+        double d[ND];
+#pragma unroll
+        for (int q = 0; q < ND; ++q) d[q] = dot[q].get();
+        block_reduce<ND>(d, red);
+        double *part = ea.partials + (size_t)j * gridDim.x * ND;
+        if (threadIdx.x < ND) part[(size_t)blockIdx.x * ND + threadIdx.x] = red[threadIdx.x];
+        double *res = ea.result + (EPI == EPI_TPQ || EPI == EPI_TAYLOR ? 0 : (size_t)FTK_HV_DOTS * j);
+        if (!last_block_reduce<ND>(part, ea.counter + j, res, red)) return;
+        if (EPI == EPI_TPQ && threadIdx.x == 0) tpq_statistics(ea, res);
+    }
+}
+
+bool gather_desc(int n, const PlanBond *bonds, int nb, double K, double J, GatherDesc *gd) {
+    if (n < 2 || n > FTK_MAX_SITES || nb < 1 || nb > 2 * FTK_MAX_PASS_BONDS) return false;
+    GatherDesc d{};
+    d.n_sites = n;
+    int w = 0;
+    for (int g = 0; g < 3; ++g) {
+        d.off[g] = w;
+        for (int q = 0; q < nb; ++q)
+            if (bonds[q].g == g) d.mask[w++] = (1u << bonds[q].i) | (1u << bonds[q].j);
+        bond_coefficients(g, K, J, &d.par[g], &d.anti[g]);
+        d.par_f[g] = (float)d.par[g];
+        d.anti_f[g] = (float)d.anti[g];
+        d.par_lo[g] = (float)(d.par[g] - (double)d.par_f[g]);
+        d.anti_lo[g] = (float)(d.anti[g] - (double)d.anti_f[g]);
+    }
+    d.off[3] = w;
+    if (w != nb) return false;
+    d.dgv[0] = J / 4;
+    d.dgv[1] = (J + K) / 4;
+    for (int c = 0; c < 2; ++c) {
+        d.dgv_f[c] = (float)d.dgv[c];
+        d.dgv_lo[c] = (float)(d.dgv[c] - (double)d.dgv_f[c]);
+    }
+    *gd = d;
+    return true;
+}
+
+// Where the line lies, us per product of B vectors, gather against the fastest
+// tiled plan (captured launches, K = -1, J = 0.1):
+//   FP64  12 sites 3.9 / 34, 16: 8.7 / 50, 18: 29 / 55, 20: 117 / 178; four
+//         vectors 4.0 / 54, 27 / 78, 107 / 156, 461 / 563: at 18 sites the
+//         gather runs at the FP64 pipe's rate
+//   FP32  12: 3.3 / 11, 16: 4.5 / 18, 18: 11 / 20, 20: 38 / 34; four vectors
+//         3.3 / 15, 10 / 19, 36 / 27, 143 / 73: from 2^19 amplitudes on the L2
+//         reads cost more than the passes
+//   DF    12: 3.7 / 17, 16: 5.8 / 25, 18: 15 / 28, 20: 53 / 65; four vectors
+//         3.7 / 67, 14 / 99, 49 / 110, 201 / 293
+bool hv_use_gather(int prec, int n, int B) {
+    if (prec != 1) return n <= 20;
+    int w = n;
+    for (int b = 1; b < B; b <<= 1) ++w;
+    return w <= 18;
+}
+
+// Threads per block: few for the smallest vectors, so that their blocks reach
+// more SMs. Blocks per column: one amplitude per thread, at most 1024 blocks
+// where their partial dots are summed by the last one.
+static int gather_threads(int n) { return n <= 12 ? 32 : n <= 14 ? 64 : 128; }
+
+template <int PREC>
+static cudaError_t launch_prec(int epi, dim3 grid, int threads, const void *in, void *out, const GatherDesc &gd,
+                               const EpiArgs &ea, cudaStream_t st) {
+    switch (epi) {
+    case EPI_PLAIN: hv_gather_kernel<PREC, EPI_PLAIN><<<grid, threads, 0, st>>>(in, out, gd, ea); break;
+    case EPI_COCG: hv_gather_kernel<PREC, EPI_COCG><<<grid, threads, 0, st>>>(in, out, gd, ea); break;
+    case EPI_COCG_MIXED:
+        if constexpr (PREC == 1) hv_gather_kernel<1, EPI_COCG_MIXED><<<grid, threads, 0, st>>>(in, out, gd, ea);
+        else return cudaErrorInvalidValue;
+        break;
+    case EPI_TPQ:
+        if constexpr (PREC == 0) hv_gather_kernel<0, EPI_TPQ><<<grid, threads, 0, st>>>(in, out, gd, ea);
+        else return cudaErrorInvalidValue;
+        break;
+    case EPI_TAYLOR:
+        if constexpr (PREC == 0) hv_gather_kernel<0, EPI_TAYLOR><<<grid, threads, 0, st>>>(in, out, gd, ea);
+        else return cudaErrorInvalidValue;
+        break;
+    default: return cudaErrorInvalidValue;
+    }
+    return cudaGetLastError();
+}
+
+cudaError_t launch_hv_gather(int prec, int B, int epi, const void *in, void *out, const GatherDesc &gd,
+                             const EpiArgs &ea, cudaStream_t st) {
+    if (B < 1 || B > FTK_MAX_RHS || ((epi == EPI_TPQ || epi == EPI_TAYLOR) && B != 1) ||
+        (epi == EPI_TAYLOR && !ea.taylor_acc) || (ea.lo && prec != 1) || (prec == 2 && ea.df_lo <= 0))
+        return cudaErrorInvalidConfiguration;
+    const int threads = gather_threads(gd.n_sites);
+    uint32_t blocks = ((1u << gd.n_sites) + threads - 1) / threads;
+    if (epi != EPI_PLAIN && blocks > 1024) blocks = 1024;
+    const dim3 grid(blocks, B);
+    const int ep = epi == EPI_COCG && ea.lo ? EPI_COCG_MIXED : epi;
+    if (prec == 0) return launch_prec<0>(ep, grid, threads, in, out, gd, ea, st);
+    if (prec == 1) return launch_prec<1>(ep, grid, threads, in, out, gd, ea, st);
+    return launch_prec<2>(ep, grid, threads, in, out, gd, ea, st);
+}
+
+}  // namespace ftk

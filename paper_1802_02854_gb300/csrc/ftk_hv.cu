@@ -59,18 +59,6 @@ struct KMask {
     static constexpr int m = (KA >= 0 ? (1 << KA) : 0) | (KB >= 0 ? (1 << KB) : 0);
 };
 
-// acc += c p for a complex amplitude and a real coefficient: on sm_100 and
-// later, float pairs take one packed FMA (fma.rn.f32x2) for both components
-__device__ __forceinline__ void cfma(double c, const double2 &p, double2 &acc) {
-    acc.x = fma(c, p.x, acc.x);
-    acc.y = fma(c, p.y, acc.y);
-}
-__device__ __forceinline__ void cfma(float c, const float2 &p, float2 &acc) {
-    acc = __ffma2_rn(make_float2(c, c), p, acc);
-}
-__device__ __forceinline__ void cadd(const double2 &p, double2 &acc) { acc.x += p.x; acc.y += p.y; }
-__device__ __forceinline__ void cadd(const float2 &p, float2 &acc) { acc = __fadd2_rn(acc, p); }
-
 // acc[k] += c(k) P[k ^ km]: c = cs where the register bits of the bond are
 // parallel (k-parity 0), cf otherwise; k, k ^ km and the choice are
 // compile-time after unrolling.
@@ -181,15 +169,9 @@ hv_pass_kernel(const typename C2<R>::t *__restrict__ in, typename C2<R>::t *out,
 #pragma unroll
         for (int k = 0; k < E; ++k) dg[k] = (R)c0[k] * d0 + (R)c1[k] * d1;
     }
-    const R scale = (EPI == EPI_TPQ) ? (R)(*ea.scale) : (R)1;
-    const R ell = (R)ea.ell, inv_n = (R)ea.inv_n;
-    // EPI_COCG_MIXED: the mixed mode's COCG epilogue; its input is the hi part
-    // of a float hi + lo residual and mu is accumulated from hi + lo with
-    // exact FMA two-products and two-sums (double-float, ~48 bits) on the
-    // FP32 pipe
-    constexpr bool MIX = EPI == EPI_COCG_MIXED;
-    constexpr int ND = (EPI == EPI_TPQ || EPI == EPI_TAYLOR) ? 2 : ((EPI == EPI_COCG || MIX) ? 2 * B : 1);
-    const R tcoef = (EPI == EPI_TAYLOR) ? (R)ea.tcoef : (R)0;
+    const HvEpilogue<R, EPI> epi(ea);
+    constexpr bool COCG = EPI == EPI_COCG || EPI == EPI_COCG_MIXED;
+    constexpr int ND = (EPI == EPI_TPQ || EPI == EPI_TAYLOR) ? 2 : (COCG ? 2 * B : 1);
     Acc<R> dot[ND];
     const bool first = pd.first != 0;
 
@@ -283,55 +265,14 @@ hv_pass_kernel(const typename C2<R>::t *__restrict__ in, typename C2<R>::t *out,
 #pragma unroll
             for (int k = 0; k < E; ++k) {
                 cx *ok = o + eofs(k);
-                if (!pd.last || EPI == EPI_PLAIN) {
+                if (!pd.last) {
 #pragma unroll
                     for (int j = 0; j < B; ++j) ok[(size_t)j * ld] = acc[k][j];
-                } else if constexpr (EPI == EPI_TPQ) {
-                    // psi' = s (l v - H v / N);  <v|Hv>, |psi'|^2
-                    const R yr = scale * (ell * pv[k][0].x - inv_n * acc[k][0].x);
-                    const R yi = scale * (ell * pv[k][0].y - inv_n * acc[k][0].y);
-                    ok[0] = mk<R>(yr, yi);
-                    dot[0].fma2(pv[k][0].x, acc[k][0].x);
-                    dot[0].fma2(pv[k][0].y, acc[k][0].y);
-                    dot[1].fma2(yr, yr);
-                    dot[1].fma2(yi, yi);
-                } else if constexpr (EPI == EPI_TAYLOR) {
-                    // cTPQ Taylor term: t' = c (l v - H v / N), acc += t';
-                    // <v|Hv> (the energy of v), |acc|^2
-                    const R yr = tcoef * (ell * pv[k][0].x - inv_n * acc[k][0].x);
-                    const R yi = tcoef * (ell * pv[k][0].y - inv_n * acc[k][0].y);
-                    ok[0] = mk<R>(yr, yi);
-                    cx *ap = reinterpret_cast<cx *>(ea.taylor_acc) + tofs + eofs(k);
-                    cx a = *ap;
-                    a.x += yr;
-                    a.y += yi;
-                    *ap = a;
-                    dot[0].fma2(pv[k][0].x, acc[k][0].x);
-                    dot[0].fma2(pv[k][0].y, acc[k][0].y);
-                    dot[1].fma2(a.x, a.x);
-                    dot[1].fma2(a.y, a.y);
-                } else if constexpr (EPI == EPI_COCG) {
-                    // W = H R;  mu_j = R_j^T W_j (bilinear)
+                } else {
 #pragma unroll
-                    for (int j = 0; j < B; ++j) {
-                        ok[(size_t)j * ld] = acc[k][j];
-                        dot[2 * j].fma2(pv[k][j].x, acc[k][j].x);
-                        dot[2 * j].fma2(-pv[k][j].y, acc[k][j].y);
-                        dot[2 * j + 1].fma2(pv[k][j].x, acc[k][j].y);
-                        dot[2 * j + 1].fma2(pv[k][j].y, acc[k][j].x);
-                    }
-                } else if constexpr (MIX) {
-                    // mixed mode: R = hi + lo, mu_j = R_j^T W_j in double-float
-#pragma unroll
-                    for (int j = 0; j < B; ++j) {
-                        ok[(size_t)j * ld] = acc[k][j];
-                        const float2 lo =
-                            reinterpret_cast<const float2 *>(ea.lo)[tofs + eofs(k) + (size_t)j * ld];
-                        dot[2 * j].fma_hl(pv[k][j].x, lo.x, acc[k][j].x);
-                        dot[2 * j].fma_hl(-pv[k][j].y, -lo.y, acc[k][j].y);
-                        dot[2 * j + 1].fma_hl(pv[k][j].x, lo.x, acc[k][j].y);
-                        dot[2 * j + 1].fma_hl(pv[k][j].y, lo.y, acc[k][j].x);
-                    }
+                    for (int j = 0; j < B; ++j)
+                        epi.apply(ea, (size_t)(tofs + eofs(k)) + (size_t)j * ld, pv[k][j], acc[k][j],
+                                  ok + (size_t)j * ld, dot + (COCG ? 2 * j : 0));
                 }
             }
         }
@@ -349,21 +290,7 @@ hv_pass_kernel(const typename C2<R>::t *__restrict__ in, typename C2<R>::t *out,
     if (threadIdx.x < ND) ea.partials[(size_t)blockIdx.x * ND + threadIdx.x] = red[threadIdx.x];
     double *res = ea.result;
     if (!last_block_reduce<ND>(ea.partials, ea.counter, res, red)) return;
-    if (EPI == EPI_TPQ && threadIdx.x == 0) {
-        // mTPQ statistics of step k (Appendix A): u_k = s^2 <v|Hv>/N,
-        // q_k = ||psi'||, <H^2>_k = N^2 (q^2 - l^2 + 2 l u_k)
-        TpqState *stt = ea.tpq;
-        const double s = stt->scale, n = stt->n_sites, l = stt->ell;
-        const double u = s * s * res[0] / n;
-        const double q2 = res[1];
-        const int k = stt->k;
-        ea.stat_u[k] = u;
-        ea.stat_logq[k] = stt->logQ;
-        ea.stat_h2[k] = n * n * (q2 - l * l + 2.0 * l * u);
-        stt->logQ += 0.5 * log(q2);
-        stt->scale = 1.0 / sqrt(q2);
-        stt->k = k + 1;
-    }
+    if (EPI == EPI_TPQ && threadIdx.x == 0) tpq_statistics(ea, res);
 }
 
 // ------------------------------------------------------------------------
@@ -376,35 +303,6 @@ hv_pass_kernel(const typename C2<R>::t *__restrict__ in, typename C2<R>::t *out,
 // part collects the rounding errors (renormalised when stored). One column
 // per launch, E = 2^LE amplitudes per thread, same tiling, groups and
 // pipeline as the kernel above.
-// The real and imaginary components take the same operations with the same
-// coefficient, so every step runs on float pairs (re, im) as one packed
-// f32x2 instruction (sm_100 and later). No step negates an operand: a - b is
-// formed as fma(b, -1, a) (the same rounding as the subtraction) and the
-// product's error term from the negated coefficient -c_hi, so each complex
-// term costs 12 packed instructions. h, l: the (re, im) hi and lo parts of
-// the accumulator.
-__device__ __forceinline__ float2 m1x2() { return make_float2(-1.f, -1.f); }
-__device__ __forceinline__ float2 fsub2(float2 a, float2 b) { return __ffma2_rn(b, m1x2(), a); }   // a - b
-// acc += c p, c = ch + cl, p = ph + pl; nch = -ch, ncl = -cl:
-//   p_hh = ch ph;  en = -(ch ph - p_hh) - ch pl - cl ph  (exact first step)
-//   t = h + p_hh, Knuth two-sum error into l together with -en
-__device__ __forceinline__ void df_acc2(float2 &h, float2 &l, float2 ch, float2 nch, float2 ncl, float2 ph, float2 pl) {
-    const float2 p = __fmul2_rn(ch, ph);
-    float2 en = __ffma2_rn(nch, ph, p);
-    en = __ffma2_rn(nch, pl, en);
-    en = __ffma2_rn(ncl, ph, en);
-    const float2 t = __fadd2_rn(h, p);
-    const float2 bb = fsub2(t, h);
-    const float2 s = __fadd2_rn(fsub2(h, fsub2(t, bb)), fsub2(p, bb));
-    l = __fadd2_rn(l, fsub2(s, en));
-    h = t;
-}
-__device__ __forceinline__ void df_add_to2(float2 &h, float2 &l, float2 ph, float2 pl) {
-    const float2 t = __fadd2_rn(h, ph);
-    const float2 bb = fsub2(t, h);
-    l = __fadd2_rn(l, __fadd2_rn(__fadd2_rn(fsub2(h, fsub2(t, bb)), fsub2(ph, bb)), pl));
-    h = t;
-}
 
 // coefficient pairs of one bond for one thread: hi, -hi, -lo of the
 // coefficient at register parity 0 (s) and 1 (f)

@@ -34,11 +34,25 @@ struct EpiArgs {
     // lowp_run (lowp NULL: always)
     const int *lowp;
     int lowp_run;
+    // COCG: the right-hand sides' seed scalars; a finished column's products are
+    // skipped (NULL: none). The gather kernel's tickets are counter[column].
+    const CocgSeed *col_seed;
     const CocgSeed *fu_seed;
     float2 *fu_rcur;
     float2 *fu_rnew;
     const float4 *fu_lam;
     double *fu_result;
+};
+
+// Bonds of the one-launch product (ftk_gather.cu), sorted by type: those of
+// type g are mask[off[g] .. off[g + 1]), with the off-diagonal amplitude par /
+// anti (parallel / antiparallel spins) of the type; dgv as in PassDesc.
+struct GatherDesc {
+    int32_t n_sites;
+    int32_t off[4];
+    uint32_t mask[2 * FTK_MAX_PASS_BONDS];
+    double par[3], anti[3], dgv[2];
+    float par_f[3], anti_f[3], par_lo[3], anti_lo[3], dgv_f[2], dgv_lo[2];
 };
 
 struct UpdArgs {
@@ -219,6 +233,11 @@ bool ctx_hamiltonian(ftk_ctx *c, CtxHam *h);
 // chunks. grid_cap bounds the persistent grid (the size of ea.partials).
 cudaError_t launch_hv_pass(int prec, int B, int epi, const void *in, void *out, const PassDesc &pd,
                            const EpiArgs &ea, int grid_cap, cudaStream_t st);
+struct PlanBond;
+bool gather_desc(int n, const PlanBond *bonds, int nb, double K, double J, GatherDesc *gd);
+bool hv_use_gather(int prec, int n, int B);
+cudaError_t launch_hv_gather(int prec, int B, int epi, const void *in, void *out, const GatherDesc &gd,
+                             const EpiArgs &ea, cudaStream_t st);
 bool hv_layout_pass(PassDesc &pd, int prec, int B);
 int hv_max_b(int prec);
 int hv_le(int prec, int B, int tile_bits, int chunk_bits);

@@ -95,12 +95,14 @@ extern "C" ftk_status ftk_tpq_step_noalloc(int32_t n_sites, const ftk_bond *bond
     NoallocScratch *s = g_scratch_ptr[dev];
     cudaStream_t st = (cudaStream_t)cuda_stream;
 
-    // plan (stack only): FP64, one vector
+    // plan (stack only): FP64, one vector; the product of a small one is one launch
+    GatherDesc gd;
+    const bool gather = hv_use_gather(0, n_sites, 1) && gather_desc(n_sites, pb, n_bonds, K, J, &gd);
     PassDesc pd[FTK_MAX_PASSES];
     int tb = 0, cb = 0;
-    const int np = plan_hv_passes(n_sites, pb, n_bonds, K, J, 16, 1, hv_max_tile_bits(0, 1), pd, FTK_MAX_PASSES,
+    const int np = gather ? 0 : plan_hv_passes(n_sites, pb, n_bonds, K, J, 16, 1, hv_max_tile_bits(0, 1), pd, FTK_MAX_PASSES,
                                   &tb, &cb);
-    if (np == 0) return noalloc_fail(FTK_EINVAL, "ftk_tpq_step_noalloc: pass planning failed");
+    if (np == 0 && !gather) return noalloc_fail(FTK_EINVAL, "ftk_tpq_step_noalloc: pass planning failed");
     for (int p = 0; p < np; ++p)
         if (!hv_layout_pass(pd[p], 0, 1)) return noalloc_fail(FTK_EINVAL, "ftk_tpq_step_noalloc: pass layout failed");
     const long grid = kNoallocMaxGrid;   // the launcher trims it to the resident CTAs
@@ -126,6 +128,10 @@ extern "C" ftk_status ftk_tpq_step_noalloc(int32_t n_sites, const ftk_bond *bond
     ea.stat_u = &s->stats[0];
     ea.stat_logq = &s->stats[1];
     ea.stat_h2 = &s->stats[2];
+    if (gather) {
+        e = launch_hv_gather(0, 1, EPI_TPQ, psi_dev, out_dev, gd, ea, st);
+        if (e != cudaSuccess) return noalloc_fail(FTK_ECUDA, cudaGetErrorString(e));
+    }
     for (int p = 0; p < np; ++p) {
         e = launch_hv_pass(0, 1, p == np - 1 ? EPI_TPQ : EPI_PLAIN, psi_dev, out_dev, pd[p], ea, (int)grid, st);
         if (e != cudaSuccess) return noalloc_fail(FTK_ECUDA, cudaGetErrorString(e));
