@@ -62,6 +62,7 @@ Layout make_layout(int n, int n_saved, int max_rhs, int prec) {
 struct Small {
     TpqState tpq;
     unsigned int counters[8];
+    unsigned int upd_counters[FTK_MAX_RHS];  // tickets of the updates' reductions, per column
     unsigned int hv_counters[FTK_MAX_RHS];   // tickets of the products' reductions, per column
     double hv_dots[FTK_MAX_RHS * FTK_HV_DOTS];
     double upd_dots[FTK_MAX_RHS * FTK_UPD_DOTS];
@@ -113,6 +114,8 @@ struct ftk_ctx {
     // shift origin of shells not produced by the mTPQ iteration (cTPQ and
     // filtered shells); NaN: an mTPQ shell, origin N u_k from the statistics
     std::vector<double> shell_origin;
+    cudaStream_t side = nullptr;           // the solve graph's branch of the shift recurrences
+    cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     cudaGraphExec_t cocg_exec = nullptr;   // instantiated COCG graph of the last solve
     std::vector<int> slot_valid;
     std::map<int, Plan> plans;       // by (precision, block width B): key prec * 64 + B
@@ -207,6 +210,15 @@ int vec_grid(ftk_ctx *ctx, uint64_t n_items) {
     const uint64_t want = (n_items + 255) / 256;
     const uint64_t cap = uint64_t(4) * ctx->n_sm;
     return (int)std::max<uint64_t>(1, std::min(want, cap));
+}
+
+// Blocks per right-hand side of the vector updates: about four resident
+// blocks per SM over all columns. (Four per SM for each column left less than
+// two amplitudes per thread at 18 sites and four columns, so that the
+// reductions at the end outweighed the elements.)
+int upd_grid(ftk_ctx *ctx, int B) {
+    const int want = vec_grid(ctx, ctx->dim);
+    return std::max(1, std::min(want, (4 * ctx->n_sm + B - 1) / B));
 }
 
 // H.V over all passes. The last pass uses epilogue epi, earlier ones write
@@ -607,9 +619,26 @@ struct IterExtras {
     const FilterAccArgs *acc;    // NULL: no accumulation
 };
 
+// The shift recurrences need only the seed scalars, and nothing but the next
+// iteration's seed kernel needs them, so they run on a branch of the captured
+// graph beside the update and the product (up to 24 us of an iteration of
+// small vectors otherwise). Fork after the seed kernel, join before the next.
+static ftk_status fork_shift(ftk_ctx *ctx, const ShiftArgs &sh, int B) {
+    CK(cudaEventRecord(ctx->ev_fork, ctx->stream));
+    CK(cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0));
+    LAUNCH(launch_cocg_shift(sh, B, ctx->side));
+    CK(cudaEventRecord(ctx->ev_join, ctx->side));
+    return FTK_OK;
+}
+
 static ftk_status cocg_iteration(ftk_ctx *ctx, int B, void *rcur, void *rprev, void *w,
                                  EpiArgs ea, const SeedArgs &sa, const ShiftArgs &sh,
-                                 UpdArgs ua, const IterExtras &ex) {
+                                 UpdArgs ua, const IterExtras &ex, bool first) {
+    // first: first iteration of the captured sequence (no branch to join yet)
+    auto join = [&]() -> ftk_status {
+        if (!first) CK(cudaStreamWaitEvent(ctx->stream, ctx->ev_join, 0));
+        return FTK_OK;
+    };
     auto after_seed = [&](void *rc, void *rp) -> ftk_status {
         if (ex.sw) {
             SwitchArgs a = *ex.sw;
@@ -634,7 +663,7 @@ static ftk_status cocg_iteration(ftk_ctx *ctx, int B, void *rcur, void *rprev, v
             u.w_lo = 0;   // w of the switching step is read without its lo part
             u.lowp = lowp;
             u.lowp_run = 1;
-            LAUNCH(launch_cocg_update(upd_kind(ctx), B, rcur, w, rprev, u, vec_grid(ctx, ctx->dim), ctx->stream));
+            LAUNCH(launch_cocg_update(upd_kind(ctx), B, rcur, w, rprev, u, upd_grid(ctx, B), ctx->stream));
             EpiArgs e1 = ea;
             e1.lo = static_cast<const char *>(rprev) + size_t(8) * ua.lo_stride;
             e1.lowp = lowp;
@@ -655,7 +684,7 @@ static ftk_status cocg_iteration(ftk_ctx *ctx, int B, void *rcur, void *rprev, v
             u.mode = 1;
             u.lowp = ea.lowp;
             u.lowp_run = 0;
-            LAUNCH(launch_cocg_update(upd_kind(ctx), B, rcur, w, rprev, u, vec_grid(ctx, ctx->dim), ctx->stream));
+            LAUNCH(launch_cocg_update(upd_kind(ctx), B, rcur, w, rprev, u, upd_grid(ctx, B), ctx->stream));
             if ((ps = run_hv(ctx, ctx->mprec, B, EPI_COCG, rprev, w, ea))) return ps;
         } else {
             ea.fu_seed = ua.seed;
@@ -664,26 +693,27 @@ static ftk_status cocg_iteration(ftk_ctx *ctx, int B, void *rcur, void *rprev, v
             ea.fu_result = ua.result;
             if ((ps = run_hv(ctx, ctx->mprec, B, EPI_COCG, rprev, w, ea))) return ps;
         }
+        ftk_status s = join();
+        if (s) return s;
         LAUNCH(launch_cocg_seed(sa, ctx->stream));
         // the new r_k is the buffer rprev (written by the update), r_{k-1} is rcur
-        ftk_status s = FTK_OK;
         if ((s = after_seed(rprev, rcur))) return s;
-        LAUNCH(launch_cocg_shift(sh, B, ctx->stream));
-        return FTK_OK;
+        return fork_shift(ctx, sh, B);
     }
     if (ctx->prec == FTK_MIXED) ea.lo = static_cast<const char *>(rcur) + size_t(8) * ua.lo_stride;
     ftk_status s = run_hv(ctx, ctx->mprec, B, EPI_COCG, rcur, w, ea);
     if (s) return s;
+    if ((s = join())) return s;
     LAUNCH(launch_cocg_seed(sa, ctx->stream));
     if ((s = after_seed(rcur, rprev))) return s;
-    LAUNCH(launch_cocg_shift(sh, B, ctx->stream));
+    if ((s = fork_shift(ctx, sh, B))) return s;
     if (ex.acc) {
         FilterAccArgs a = *ex.acc;
         a.r = static_cast<const double2 *>(rcur);
         LAUNCH(launch_filter_acc(a, vec_grid(ctx, ctx->dim), ctx->stream));
     }
     ua.mode = 1;
-    LAUNCH(launch_cocg_update(upd_kind(ctx), B, rcur, w, rprev, ua, vec_grid(ctx, ctx->dim), ctx->stream));
+    LAUNCH(launch_cocg_update(upd_kind(ctx), B, rcur, w, rprev, ua, upd_grid(ctx, B), ctx->stream));
     return FTK_OK;
 }
 
@@ -793,7 +823,7 @@ static ftk_status cocg_core(ftk_ctx *ctx, const CocgReq &rq, double *G_out, int3
     }
     ua.seed = d->seed;
     ua.partials = (double *)wsp(ctx, ctx->L.partials);
-    ua.counter = &d->counters[3];
+    ua.counter = d->upd_counters;
     ua.result = d->upd_dots;
     ua.all_done = &d->all_done;
     ua.lo_stride = (long long)ctx->max_rhs * (long long)ctx->dim;   // mixed and double-float modes
@@ -852,7 +882,7 @@ static ftk_status cocg_core(ftk_ctx *ctx, const CocgReq &rq, double *G_out, int3
         CK(cudaMemsetAsync(rprev, 0, ctx->L.vec_bytes * B, ctx->stream));
     }
     ua.mode = 0;
-    LAUNCH(launch_cocg_update(upd_kind(ctx), B, nullptr, nullptr, rcur, ua, vec_grid(ctx, ctx->dim), ctx->stream));
+    LAUNCH(launch_cocg_update(upd_kind(ctx), B, nullptr, nullptr, rcur, ua, upd_grid(ctx, B), ctx->stream));
     int it0 = 0;
     if (ctx->prec == FTK_DF) {
         // step 0 without the fused update: W = H r_0 (+mu), seed, shifts
@@ -864,7 +894,15 @@ static ftk_status cocg_core(ftk_ctx *ctx, const CocgReq &rq, double *G_out, int3
         it0 = 1;
     }
 
-    // Capture two iterations (buffer roles return to the start) in a graph.
+    // Capture four iterations (an even number: buffer roles return to the
+    // start; the last one's shift branch is the only one without work beside
+    // it) in a graph.
+    const int per_launch = 4;
+    if (!ctx->side) {
+        CK(cudaStreamCreateWithFlags(&ctx->side, cudaStreamNonBlocking));
+        CK(cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming));
+        CK(cudaEventCreateWithFlags(&ctx->ev_join, cudaEventDisableTiming));
+    }
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     const int64_t l0 = ctx->launches;
@@ -873,8 +911,11 @@ static ftk_status cocg_core(ftk_ctx *ctx, const CocgReq &rq, double *G_out, int3
     {
         std::lock_guard<std::mutex> lk(device_mu());
         CK(cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal));
-        ftk_status cs = cocg_iteration(ctx, B, rcur, rprev, w, ea, sa, sh, ua, ex);
-        if (cs == FTK_OK) cs = cocg_iteration(ctx, B, rprev, rcur, w, ea, sa, sh, ua, ex);
+        ftk_status cs = FTK_OK;
+        for (int q = 0; q < per_launch && cs == FTK_OK; ++q)
+            cs = cocg_iteration(ctx, B, (q & 1) ? rprev : rcur, (q & 1) ? rcur : rprev, w, ea, sa, sh, ua, ex, q == 0);
+        if (cs == FTK_OK && cudaStreamWaitEvent(ctx->stream, ctx->ev_join, 0) != cudaSuccess)
+            cs = fail(ctx, FTK_ECUDA, "joining the shift branch of the solve graph");
         ce = cudaStreamEndCapture(ctx->stream, &graph);
         if (cs != FTK_OK) { if (graph) cudaGraphDestroy(graph); return cs; }
         CK(ce);
@@ -885,10 +926,10 @@ static ftk_status cocg_core(ftk_ctx *ctx, const CocgReq &rq, double *G_out, int3
         if (is != FTK_OK) return is;
     }
     int done = 0, it = it0;
-    const int chunk = 16;   // graph launches between host checks (32 iterations)
+    const int chunk = 32 / per_launch;   // graph launches between host checks
     ftk_status result = FTK_OK;
     while (!done) {
-        for (int g = 0; g < chunk && it <= rq.max_iter + 2; ++g, it += 2) {
+        for (int g = 0; g < chunk && it <= rq.max_iter + 2; ++g, it += per_launch) {
             ce = cudaGraphLaunch(exec, ctx->stream);
             if (ce != cudaSuccess) break;
             ctx->launches += per_graph;
@@ -1579,6 +1620,9 @@ void ftk_destroy(ftk_ctx *ctx) {
     if (ctx->slot_energy) cudaFree(ctx->slot_energy);
     if (ctx->slot_norm2) cudaFree(ctx->slot_norm2);
     if (ctx->cocg_exec) cudaGraphExecDestroy(ctx->cocg_exec);
+    if (ctx->ev_fork) cudaEventDestroy(ctx->ev_fork);
+    if (ctx->ev_join) cudaEventDestroy(ctx->ev_join);
+    if (ctx->side) cudaStreamDestroy(ctx->side);
     if (ctx->own_stream && ctx->stream) cudaStreamDestroy(ctx->stream);
     delete ctx;
 }

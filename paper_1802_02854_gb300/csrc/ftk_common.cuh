@@ -85,6 +85,8 @@ struct CocgSeed {
     double rho_prev_re, rho_prev_im;
     double alpha_re, alpha_im;  // alpha_k
     double alpha_prev_re, alpha_prev_im;
+    double irho_re, irho_im;      // 1 / rho_k
+    double ialpha_re, ialpha_im;  // 1 / alpha_k
     double beta_prev_re, beta_prev_im;  // beta_{k-1}
     double c_re, c_im;          // c_k = beta_{k-1} alpha_k / alpha_{k-1}
     double a1_re, a1_im;        // 1 + c_k - alpha_k z_s: coefficient of r_k in r_{k+1}

@@ -73,10 +73,41 @@ template <> struct Acc<float> {
 };
 
 // ---------------------------------------------------------- reductions
-__device__ __forceinline__ double warp_sum(double v) {
+// Sums of ND <= 8 values over a warp: the values are folded over the lanes
+// (at each of the first levels a lane keeps one half of its values and hands
+// the other half over), so 5 values take 9 additions per lane instead of 25;
+// on this chip's FP64 pipe (2 lanes per clock and SM) the plain butterfly
+// cost a vector kernel of few elements per thread as much as its own work.
+// On return lane l holds the sum of value warp_sums_index<ND>(l).
+template <int ND>
+struct WarpFold {
+    static constexpr int P = ND > 4 ? 8 : ND > 2 ? 4 : ND > 1 ? 2 : 1;   // values, padded with zeros
+    static constexpr int levels = P == 8 ? 3 : P == 4 ? 2 : P == 2 ? 1 : 0;
+};
+template <int ND>
+__device__ __forceinline__ int warp_sums_index(int lane) { return lane >> (5 - WarpFold<ND>::levels); }
+template <int ND>
+__device__ __forceinline__ double warp_sums(const double (&v)[ND]) {
+    static_assert(ND >= 1 && ND <= 8, "");
+    constexpr int P = WarpFold<ND>::P;
+    const int lane = threadIdx.x & 31;
+    double a[P];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
+    for (int d = 0; d < P; ++d) a[d] = d < ND ? v[d] : 0.0;
+    int o = 16;
+#pragma unroll
+    for (int h = P / 2; h >= 1; h /= 2, o /= 2) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int d = 0; d < P / 2; ++d)
+            if (d < h) {
+                const double keep = up ? a[d + h] : a[d], give = up ? a[d] : a[d + h];
+                a[d] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+            }
+    }
+#pragma unroll
+    for (; o > 0; o /= 2) a[0] += __shfl_xor_sync(0xffffffffu, a[0], o);
+    return a[0];
 }
 
 // Reduce nd values per thread over the block (fixed order) into red[0..nd).
@@ -85,12 +116,21 @@ __device__ __forceinline__ double warp_sum(double v) {
 template <int ND>
 __device__ void block_reduce(double (&v)[ND], double *red) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    constexpr int NG = ND <= 8 ? ND : 8;   // values folded at a time
+    static_assert(ND % NG == 0, "");
+    double s[ND / NG];
 #pragma unroll
-    for (int d = 0; d < ND; ++d) v[d] = warp_sum(v[d]);
+    for (int g = 0; g < ND / NG; ++g) {
+        double a[NG];
+#pragma unroll
+        for (int d = 0; d < NG; ++d) a[d] = v[g * NG + d];
+        s[g] = warp_sums<NG>(a);
+    }
+    const int d = warp_sums_index<NG>(lane);
     __syncthreads();
-    if (lane == 0) {
+    if (d < NG && (lane & ((1 << (5 - WarpFold<NG>::levels)) - 1)) == 0) {
 #pragma unroll
-        for (int d = 0; d < ND; ++d) red[warp * ND + d] = v[d];
+        for (int g = 0; g < ND / NG; ++g) red[warp * ND + g * NG + d] = s[g];
     }
     __syncthreads();
     if (threadIdx.x < ND) {

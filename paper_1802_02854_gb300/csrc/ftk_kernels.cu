@@ -117,25 +117,10 @@ __global__ void __launch_bounds__(256) cocg_update_kernel(V vec, UpdArgs ua) {
     }
     double v[5] = {d_rr.get(), d_ri.get(), d_gr.get(), d_gi.get(), d_n.get()};
     block_reduce<5>(v, red);
-    const unsigned nblk = gridDim.x * gridDim.y;
-    double *part = ua.partials + ((size_t)j * gridDim.x + blockIdx.x) * 5;
-    if (threadIdx.x < 5) part[threadIdx.x] = red[threadIdx.x];
-    // last block: fixed-order sum of the partials -> ua.result[B][FTK_UPD_DOTS]
-    __shared__ int am_last;
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) am_last = (atomicAdd(ua.counter, 1u) == nblk - 1);
-    __syncthreads();
-    if (!am_last) return;
-    __threadfence();
-    for (int q = threadIdx.x; q < (int)gridDim.y * 5; q += blockDim.x) {
-        const int jj = q / 5, d = q % 5;
-        double sum = 0.0;
-        for (unsigned bb = 0; bb < gridDim.x; ++bb)
-            sum += __ldcg(ua.partials + ((size_t)jj * gridDim.x + bb) * 5 + d);
-        ua.result[jj * FTK_UPD_DOTS + d] = sum;
-    }
-    if (threadIdx.x == 0) *ua.counter = 0u;
+    // the column's last block: fixed-order sum of its partials
+    double *part = ua.partials + (size_t)j * gridDim.x * 5;
+    if (threadIdx.x < 5) part[(size_t)blockIdx.x * 5 + threadIdx.x] = red[threadIdx.x];
+    last_block_reduce<5>(part, ua.counter + j, ua.result + j * FTK_UPD_DOTS, red);
 }
 
 // Mixed and double-float modes: the residuals r_k, r_{k-1} (float hi + lo
@@ -196,25 +181,10 @@ cocg_update_df_kernel(float2 *rcur, const float2 *__restrict__ w, float2 *rnew, 
     double v[5];
     dots.get(v);
     block_reduce<5>(v, red);
-    const unsigned nblk = gridDim.x * gridDim.y;
-    double *part = ua.partials + ((size_t)j * gridDim.x + blockIdx.x) * 5;
-    if (threadIdx.x < 5) part[threadIdx.x] = red[threadIdx.x];
-    // last block: fixed-order sum of the partials -> ua.result[B][FTK_UPD_DOTS]
-    __shared__ int am_last;
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) am_last = (atomicAdd(ua.counter, 1u) == nblk - 1);
-    __syncthreads();
-    if (!am_last) return;
-    __threadfence();
-    for (int q = threadIdx.x; q < (int)gridDim.y * 5; q += blockDim.x) {
-        const int jj = q / 5, d = q % 5;
-        double sum = 0.0;
-        for (unsigned bb = 0; bb < gridDim.x; ++bb)
-            sum += __ldcg(ua.partials + ((size_t)jj * gridDim.x + bb) * 5 + d);
-        ua.result[jj * FTK_UPD_DOTS + d] = sum;
-    }
-    if (threadIdx.x == 0) *ua.counter = 0u;
+    // the column's last block: fixed-order sum of its partials
+    double *part = ua.partials + (size_t)j * gridDim.x * 5;
+    if (threadIdx.x < 5) part[(size_t)blockIdx.x * 5 + threadIdx.x] = red[threadIdx.x];
+    last_block_reduce<5>(part, ua.counter + j, ua.result + j * FTK_UPD_DOTS, red);
 }
 
 // ------------------------------------------------------------ seed scalars
@@ -239,25 +209,41 @@ __device__ __forceinline__ dcx cdiv(dcx a, dcx b) {
 }
 __device__ __forceinline__ double cabs_(dcx a) { return hypot(a.re, a.im); }
 
+// |a| against a bound far from the extremes of the range: no square root
+__device__ __forceinline__ double cmax_(dcx a) { return fmax(fabs(a.re), fabs(a.im)); }
+// 1 / a: the plain quotient where |a|^2 neither overflows nor loses digits,
+// Smith's algorithm elsewhere
+__device__ __forceinline__ dcx cinv(dcx a, double *n2_inv) {
+    const double n2 = fma(a.re, a.re, a.im * a.im);
+    *n2_inv = 1.0 / n2;
+    if (n2 > 1e-280 && n2 < 1e280) return {a.re * *n2_inv, -a.im * *n2_inv};
+    const double m = cabs_(a);
+    *n2_inv = 1.0 / m / m;
+    return cdiv({1.0, 0.0}, a);
+}
+
+// One thread per right-hand side, on a copy of its scalars in registers: the
+// launch is a chain of dependent FP64 operations and nothing else, so its
+// time is the chain's length. Of the three complex quotients of the textbook
+// form only 1 / denom is on it; 1 / rho_k (for beta of the next step) runs
+// beside it, and 1 / alpha_k = denom / rho_k follows from both.
 __global__ void cocg_seed_kernel(SeedArgs sa) {
     const int j = threadIdx.x;
+    int done = 1, small = 1;
     if (j < sa.n_rhs) {
-        CocgSeed &s = sa.seed[j];
+        CocgSeed s = sa.seed[j];
         s.sw = 0;
         if (!s.done) seed_one(sa, s, j);
+        sa.seed[j] = s;
+        done = s.done != 0;
+        if (!done) small = s.k >= 2 && s.resid < sa.relax;   // resid set from k = 1 on
     }
-    __syncthreads();
+    const int all = __all_sync(0xffffffffu, done), every = __all_sync(0xffffffffu, small);
     if (threadIdx.x == 0) {
-        int all = 1, small = 1;
-        for (int q = 0; q < sa.n_rhs; ++q) {
-            const CocgSeed &s = sa.seed[q];
-            all &= (s.done != 0);
-            if (!s.done) small &= (s.k >= 2 && s.resid < sa.relax);   // resid set from k = 1 on
-        }
         *sa.all_done = all;
         // relaxed solve: from here on the matrix-vector products may run in
         // FP32 (their errors enter scaled by the small residual)
-        if (sa.lowp && sa.relax > 0.0 && small && !all) *sa.lowp = 1;
+        if (sa.lowp && sa.relax > 0.0 && every && !all) *sa.lowp = 1;
     }
 }
 
@@ -315,8 +301,12 @@ __device__ void seed_one(const SeedArgs &sa, CocgSeed &s, int j) {
             nrm *= cabs_(s1);
             const dcx rp = cmul({s.rho_re, s.rho_im}, s0s);
             s.rho_re = rp.re; s.rho_im = rp.im;
+            const dcx irp = cdiv(one, rp);
+            s.irho_re = irp.re; s.irho_im = irp.im;
             const dcx ap = cmul({s.alpha_re, s.alpha_im}, cdiv(s1, s0));
             s.alpha_re = ap.re; s.alpha_im = ap.im;
+            const dcx iap = cdiv(one, ap);
+            s.ialpha_re = iap.re; s.ialpha_im = iap.im;
             s.zs_re = s.e0 + sa.shift[best].re;
             s.zs_im = sa.shift[best].im;
             s.seed_idx = best;
@@ -328,22 +318,22 @@ __device__ void seed_one(const SeedArgs &sa, CocgSeed &s, int j) {
     // r^T r vanished: at a residual 1e-12 below ||lambda|| this is the
     // underflow of FP32 vectors (the seed system is solved far beyond any
     // shifted one can still gain): stop as converged; otherwise a breakdown
-    if (cabs_(rho) <= 1e-300 * (nrm * nrm)) { s.done = nrm <= 1e-12 * s.lnorm ? 1 : 2; return; }
+    if (cmax_(rho) <= 1e-300 * (nrm * nrm)) { s.done = nrm <= 1e-12 * s.lnorm ? 1 : 2; return; }
     dcx zs = {s.zs_re, s.zs_im};
     dcx beta = {0, 0}, c = {0, 0};
-    dcx denom = {cmul(zs, rho).re - mu.re, cmul(zs, rho).im - mu.im};
+    const dcx zr = cmul(zs, rho);
+    dcx denom = {zr.re - mu.re, zr.im - mu.im};
     if (k >= 1) {
-        dcx rp = {s.rho_re, s.rho_im}, ap = {s.alpha_re, s.alpha_im};
-        beta = cdiv(rho, rp);
-        dcx t = cdiv(cmul(beta, rho), ap);
+        beta = cmul(rho, {s.irho_re, s.irho_im});
+        const dcx t = cmul(cmul(beta, rho), {s.ialpha_re, s.ialpha_im});
         denom.re -= t.re; denom.im -= t.im;
     }
-    if (cabs_(denom) == 0.0) { s.done = 3; return; }
-    dcx alpha = cdiv(rho, denom);
-    if (k >= 1) {
-        dcx ap = {s.alpha_re, s.alpha_im};
-        c = cdiv(cmul(beta, alpha), ap);
-    }
+    if (cmax_(denom) == 0.0) { s.done = 3; return; }
+    double n2;
+    const dcx irho = cinv(rho, &n2), iden = cinv(denom, &n2);
+    const dcx alpha = cmul(rho, iden);
+    if (k >= 1) c = cmul(cmul(beta, alpha), {s.ialpha_re, s.ialpha_im});
+    const dcx ialpha = cmul(denom, irho);
     // Range guard: the seed residual can fall many orders below ||lambda||
     // while slow shifts still converge (their |pi| falls with it); FP32 and
     // float-pair storage would underflow. Every quantity of the recurrences
@@ -355,6 +345,9 @@ __device__ void seed_one(const SeedArgs &sa, CocgSeed &s, int j) {
     s.rescale = f;
     s.rho_prev_re = s.rho_re; s.rho_prev_im = s.rho_im;
     s.rho_re = rho.re * f * f; s.rho_im = rho.im * f * f;
+    const double f2 = 1.0 / (f * f);   // a power of two: exact
+    s.irho_re = irho.re * f2; s.irho_im = irho.im * f2;
+    s.ialpha_re = ialpha.re; s.ialpha_im = ialpha.im;
     s.alpha_prev_re = s.alpha_re; s.alpha_prev_im = s.alpha_im;
     s.alpha_re = alpha.re; s.alpha_im = alpha.im;
     s.beta_prev_re = beta.re; s.beta_prev_im = beta.im;
@@ -374,60 +367,62 @@ __device__ void seed_one(const SeedArgs &sa, CocgSeed &s, int j) {
 //   pi_{k+1}     = (1 + alpha_k D) pi_k + c_k (pi_k - pi_{k-1})
 //   alpha^s_k    = alpha_k pi_k / pi_{k+1},   G^s += alpha^s_k p~^s_k
 // and the per-RHS max of 1/|pi_{k+1}| for the next convergence test.
-__global__ void cocg_shift_kernel(ShiftArgs sh) {
+// Blocks of one warp: the recurrences are bound by the FP64 pipe of the SMs
+// they run on (256 shifts in one block took 24 us on one SM), and 1 / pi_k,
+// 1 / pi_{k+1} are formed once each instead of four quotients and a hypot.
+__global__ void __launch_bounds__(32) cocg_shift_kernel(ShiftArgs sh) {
     const int j = blockIdx.y;
     const int si = blockIdx.x * blockDim.x + threadIdx.x;
     const CocgSeed &s = sh.seed[j];
-    __shared__ double wmax[256 / 32];
-    double inv_pi = 0.0;
-    bool active = (si < sh.n_omega) && !s.done;
+    double inv_pi2 = 0.0;   // 1 / |pi_{k+1}|^2
+    const int done = s.done;
+    bool active = (si < sh.n_omega) && !done;
     const size_t o = (size_t)j * sh.n_omega + si;
     if (active && sh.frozen[o]) active = false;
+    dcx pc = {1.0, 0.0};
     if (active) {
         // freeze a shift whose residual ||r_k|| / |pi_k| reached tol ||lambda||
-        const dcx pc0 = sh.pi_cur[o];
-        if (s.nrm <= sh.tol * s.lnorm * cabs_(pc0)) { sh.frozen[o] = 1; active = false; }
+        pc = sh.pi_cur[o];
+        if (s.nrm <= sh.tol * s.lnorm * sqrt(fma(pc.re, pc.re, pc.im * pc.im))) { sh.frozen[o] = 1; active = false; }
     }
     // history (right-hand side 0): iteration k = s.k - 1 of a running solve
-    const int kh = s.k - 1;
-    dcx* hrec = (sh.hist && j == 0 && !s.done && si < sh.n_omega && kh >= 0 && kh < sh.hist_cap)
-                    ? sh.hist + ((size_t)kh * sh.n_omega + si) * 3 : nullptr;
+    const int k = s.k - 1;   // iteration just computed by the seed kernel
+    dcx* hrec = (sh.hist && j == 0 && !done && si < sh.n_omega && k >= 0 && k < sh.hist_cap)
+                    ? sh.hist + ((size_t)k * sh.n_omega + si) * 3 : nullptr;
     if (hrec) { hrec[0] = {0.0, 0.0}; hrec[1] = {0.0, 0.0}; hrec[2] = {0.0, 0.0}; }
     if (active) {
-        const int k = s.k - 1;   // iteration just computed by the seed kernel
-        dcx pc = sh.pi_cur[o], pp = sh.pi_prev[o], pt = sh.ptil[o], G = sh.G[o];
+        const dcx pp = sh.pi_prev[o];
+        dcx pt = sh.ptil[o], G = sh.G[o];
         const dcx alpha = {s.alpha_re, s.alpha_im}, c = {s.c_re, s.c_im};
         const dcx beta = {s.beta_prev_re, s.beta_prev_im}, g = {s.g_re, s.g_im};
         const dcx zs = sh.shift[s.seed_idx], zo = sh.shift[si];
         const dcx D = {zo.re - zs.re, zo.im - zs.im};
-        dcx bs = {0, 0};
-        if (k >= 1) { dcx r = cdiv(pp, pc); bs = cmul(cmul(r, r), beta); }
-        dcx gp = cdiv(g, pc), bp = cmul(bs, pt);
-        pt = {gp.re + bp.re, gp.im + bp.im};
-        dcx aD = cmul(alpha, D);
-        dcx t1 = cmul({1.0 + aD.re, aD.im}, pc);
-        dcx t2 = cmul(c, {pc.re - pp.re, pc.im - pp.im});
+        double n2;
+        const dcx ipc = cinv(pc, &n2);
+        const dcx aD = cmul(alpha, D);
+        const dcx t1 = cmul({1.0 + aD.re, aD.im}, pc);
+        const dcx t2 = cmul(c, {pc.re - pp.re, pc.im - pp.im});
         dcx pn = {t1.re + t2.re, t1.im + t2.im};
-        dcx as = cdiv(cmul(alpha, pc), pn);
-        dcx ag = cmul(as, pt);
+        const dcx ipn = cinv(pn, &inv_pi2);
+        dcx bs = {0, 0};
+        if (k >= 1) { const dcx r = cmul(pp, ipc); bs = cmul(cmul(r, r), beta); }
+        const dcx gp = cmul(g, ipc), bp = cmul(bs, pt);
+        pt = {gp.re + bp.re, gp.im + bp.im};
+        const dcx as = cmul(cmul(alpha, pc), ipn);
+        const dcx ag = cmul(as, pt);
         G.re += ag.re; G.im += ag.im;
-        if (hrec) { hrec[0] = as; hrec[1] = bs; hrec[2] = cdiv({1.0, 0.0}, pc); }
+        if (hrec) { hrec[0] = as; hrec[1] = bs; hrec[2] = ipc; }
         const double f = s.rescale;   // range guard of the seed kernel (1 or a power of two)
         pc.re *= f; pc.im *= f; pn.re *= f; pn.im *= f;
+        inv_pi2 /= f * f;
         sh.pi_prev[o] = pc; sh.pi_cur[o] = pn; sh.ptil[o] = pt; sh.G[o] = G;
-        inv_pi = 1.0 / cabs_(pn);
     }
-    // block max -> atomicMax on the (non-negative) double's bit pattern
+    // warp max -> atomicMax on the (non-negative) double's bit pattern
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) inv_pi = fmax(inv_pi, __shfl_xor_sync(0xffffffffu, inv_pi, o));
-    if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = inv_pi;
-    __syncthreads();
-    if (threadIdx.x == 0 && !s.done) {
-        double m = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) m = fmax(m, wmax[w]);
+    for (int q = 16; q > 0; q >>= 1) inv_pi2 = fmax(inv_pi2, __shfl_xor_sync(0xffffffffu, inv_pi2, q));
+    if (threadIdx.x == 0 && !done)
         atomicMax(reinterpret_cast<unsigned long long *>(sh.inv_pi_max + ((s.k & 1) * FTK_MAX_RHS) + j),
-                  (unsigned long long)__double_as_longlong(m));
-    }
+                  (unsigned long long)__double_as_longlong(sqrt(inv_pi2)));
 }
 
 // ------------------------------------------------------------ seed switch
@@ -834,8 +829,8 @@ cudaError_t launch_cocg_seed(const SeedArgs &sa, cudaStream_t st) {
 }
 
 cudaError_t launch_cocg_shift(const ShiftArgs &sh, int n_rhs, cudaStream_t st) {
-    dim3 grid((sh.n_omega + 255) / 256, n_rhs);
-    cocg_shift_kernel<<<grid, 256, 0, st>>>(sh);
+    dim3 grid((sh.n_omega + 31) / 32, n_rhs);
+    cocg_shift_kernel<<<grid, 32, 0, st>>>(sh);
     return cudaGetLastError();
 }
 
