@@ -141,23 +141,25 @@ __device__ void block_reduce(double (&v)[ND], double *red) {
     __syncthreads();
 }
 
-// Called by every thread of every CTA after it stored its ND partials at
-// partials[blockIdx.x * ND + d]. Returns true in the (unique) last CTA, after
-// it reduced all partials into out[0..ND) in a fixed order. Resets counter.
+// Called by every thread of the nblk CTAs of a sum (the whole grid row if 0)
+// after each stored its ND partials at partials[block * ND + d]. Returns true
+// in the (unique) last CTA, after it reduced all partials into out[0..ND) in a
+// fixed order. Resets counter.
 template <int ND>
 __device__ bool last_block_reduce(const double *partials, unsigned int *counter, double *out,
-                                  double *red) {
+                                  double *red, unsigned int nblk = 0) {
+    if (nblk == 0) nblk = gridDim.x;
     __shared__ int am_last;
     __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0) am_last = (atomicAdd(counter, 1u) == gridDim.x - 1);
+    if (threadIdx.x == 0) am_last = (atomicAdd(counter, 1u) == nblk - 1);
     __syncthreads();
     if (!am_last) return false;
     __threadfence();
     double v[ND];
 #pragma unroll
     for (int d = 0; d < ND; ++d) v[d] = 0.0;
-    for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) {
+    for (int b = threadIdx.x; b < (int)nblk; b += blockDim.x) {
 #pragma unroll
         for (int d = 0; d < ND; ++d) v[d] += __ldcg(partials + (size_t)b * ND + d);
     }

@@ -16,10 +16,11 @@
 // output representative:
 //   (H v)_r' = D(r') v_r' + sum_b c_b(r') chi(g_b)^* sqrt(o_r' / o_r'') v_r'',
 //   r'' = rep(flip_b r'), flip_b r' = g_b . r''.
-// Data on the device: loc[x] = (orbit index << 5) | g for every state x
-// (g . rep = x), the representatives and stabiliser masks of all orbits, and
-// per sector the map orbit -> sector index (-1 where chi is not 1 on the
-// stabiliser) and sqrt(o) per sector index. FP64 complex sector vectors.
+// Data on the device: for every state x the sector index of its orbit and the
+// element g with g . rep = x (loc[x], see kLocNone), the representatives and
+// stabiliser masks of all orbits, and per sector the map orbit -> sector index
+// (-1 where chi is not 1 on the stabiliser), the representative and sqrt(o)
+// per sector index. FP64 complex sector vectors.
 //
 // The sector Hamiltonian is complex Hermitian, not real symmetric, so the
 // bilinear COCG of the full basis does not apply; the Green's function of a
@@ -152,11 +153,22 @@ __global__ void __launch_bounds__(kSecThreads) sec_compact_kernel(SecGroup G, ui
     }
 }
 
-// loc[x] = orbit index * 32 + g (unsigned: up to 2^27 orbits)
+// loc[x] = sector index * 32 + g of a state whose orbit is in the sector,
+// kLocNone of the others. Groups of at most 16 elements leave bit 4 of g free;
+// it marks the orbits of full size (nearly all), whose sqrt(o) ratio is 1.
+constexpr uint32_t kLocNone = 0xffffffffu;
+constexpr uint32_t kLocFull = 16u;
 __global__ void sec_loc_kernel(uint64_t dim, const uint32_t *rep_of, const uint8_t *g_of, const int32_t *idx_of,
-                               uint32_t *loc) {
-    for (uint64_t x = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; x < dim; x += (uint64_t)gridDim.x * blockDim.x)
-        loc[x] = ((uint32_t)idx_of[rep_of[x]] << 5) | (uint32_t)g_of[x];
+                               const int32_t *sec_index, const uint32_t *orb_stab, int flag_full, uint32_t *loc) {
+    for (uint64_t x = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; x < dim; x += (uint64_t)gridDim.x * blockDim.x) {
+        const int32_t o = idx_of[rep_of[x]], i = sec_index[o];
+        uint32_t L = kLocNone;
+        if (i >= 0) {
+            L = ((uint32_t)i << 5) | (uint32_t)g_of[x];
+            if (flag_full && orb_stab[o] == 1u) L |= kLocFull;
+        }
+        loc[x] = L;
+    }
 }
 
 // sector basis: the orbits on whose stabiliser chi is 1 (flag, then compaction
@@ -171,113 +183,260 @@ __global__ void sec_valid_kernel(int n_orb, int ng, const uint32_t *orb_stab, co
     }
 }
 
-__global__ void sec_fill_kernel(int n_orb, int ng, const uint32_t *orb_stab, const int *flag, const int *pos,
-                                int32_t *sec_index, int32_t *sec_orbit, double *sqo) {
+__global__ void sec_fill_kernel(int n_orb, int ng, const uint32_t *orb_rep, const uint32_t *orb_stab, const int *flag,
+                                const int *pos, int32_t *sec_index, int32_t *sec_orbit, uint32_t *sec_rep, double *sqo) {
     for (int o = blockIdx.x * blockDim.x + threadIdx.x; o < n_orb; o += gridDim.x * blockDim.x) {
         if (!flag[o]) { sec_index[o] = -1; continue; }
         const int i = pos[o];
         sec_index[o] = i;
         sec_orbit[i] = o;
+        sec_rep[i] = orb_rep[o];
         sqo[i] = sqrt((double)ng / (double)__popc(orb_stab[o]));
     }
 }
 
 // ---------------------------------------------------------------- sector H.v
+// A bond's type and parity select one of six real amplitudes; bonds sorted by
+// type, those of type g in [off[g], off[g + 1]).
 struct SecHam {
-    int nb;
+    int off[4];
     uint32_t mask[2 * FTK_MAX_PASS_BONDS];
-    uint8_t bi[2 * FTK_MAX_PASS_BONDS];
-    double par[2 * FTK_MAX_PASS_BONDS], anti[2 * FTK_MAX_PASS_BONDS], dg[2 * FTK_MAX_PASS_BONDS];
+    double c[6];               // 2 g + odd: parallel / antiparallel amplitude of type g
+    double dgv[2];             // diagonal of the x and y bonds, and of the z bonds
 };
 
 enum { SEC_PLAIN = 0, SEC_TPQ = 1, SEC_DOT = 2 };
 
+// Scalars of iteration j of the Lanczos process: a_j, b_{j+1} and the inverse
+// norms 1 / b_j of its vectors (kept unnormalised) in rings of four; per shift
+// 1 / d_j, y_j, G, frozen once |b_{j+1} y_j / d_j| <= tol; done when every
+// shift is frozen, b_{j+1} vanished, or j + 1 = max_iter.
+struct LzShiftArgs {
+    int n_shift, n_blocks, max_iter, j;
+    double tol;
+    const double2 *z;          // [n_shift]
+    const double *alpha;       // a_j
+    const double *beta;        // b_j
+    const double *beta_next;   // b_{j+1}
+    double2 *id, *y, *G;       // [n_shift]
+    int *frozen;               // [n_shift]
+    int *iter;                 // j + 1 once evaluated
+    int *done;                 // 0, or 4 (j + 1) + 1 (every shift frozen) or + 2 (max_iter)
+    unsigned int *counter;     // [2]: ticket, shifts still running
+};
+
 struct SecHvArgs {
     int64_t dim;
     const uint32_t *loc;
-    const uint32_t *orb_rep;
-    const int32_t *sec_index, *sec_orbit;
+    const uint32_t *rep;      // [dim]
     const double *sqo;
+    double full;              // sqrt(o) of an orbit of full size
+    int flag_full, ng;        // loc marks them (kLocFull); group elements
     const double2 *chi;       // [ng]
     const double2 *in;
     double2 *out;
     double ell, inv_n;        // SEC_TPQ: out = ell v - H v / N
     const double *in_scale;   // optional device scale of the input (NULL: 1)
-    double *partials;         // [grid][3]
+    double *partials;         // [grid][2]
     unsigned int *counter;
-    double *result;           // [3]: <v|Hv>, |out|^2, |v|^2 (SEC_TPQ / SEC_DOT)
+    double *result;           // SEC_DOT: <v|Hv>
+    // SEC_TPQ: <v|Hv> and |out|^2 of the step, and 1 / |out| for the next one
+    double *stat_e, *stat_q2, *next_scale;
+    LzShiftArgs lz;           // shift recurrences of the previous iteration (lz.n_blocks leading blocks)
+    // SEC_DOT: nothing to do once set by the shifts of an earlier launch (those
+    // of this launch belong to iteration iter - 1; NULL: always run). All
+    // blocks decide alike, whenever they start.
+    const int *done;
+    int iter;
 };
 
+// 1 / a: the plain quotient inside the range of |a|^2, Smith's algorithm outside
+__device__ __forceinline__ dcx zinv(dcx a) {
+    const double n2 = fma(a.re, a.re, a.im * a.im);
+    if (n2 > 1e-280 && n2 < 1e280) {
+        const double q = 1.0 / n2;
+        return {a.re * q, -a.im * q};
+    }
+    return zdiv({1.0, 0.0}, a);
+}
+
+constexpr int kShiftsPerBlock = 32;
+
+// One block of the shift recurrences of iteration a.j (block b of a.n_blocks).
+__device__ void lz_shift_block(const LzShiftArgs &a, int b) {
+    const int s = b * kShiftsPerBlock + threadIdx.x;
+    const double bn = *a.beta_next;
+    int running = 0;
+    if (threadIdx.x < kShiftsPerBlock && s < a.n_shift && !a.frozen[s]) {
+        const double al = *a.alpha, bj = *a.beta;
+        const double2 z = a.z[s];
+        dcx dn = {z.x - al, z.y}, yn = {1.0, 0.0};
+        if (a.j > 0) {
+            const double2 ip = a.id[s], yp = a.y[s];
+            const dcx t = {bj * ip.x, bj * ip.y};   // b_j / d_{j-1}
+            dn.re -= bj * t.re;
+            dn.im -= bj * t.im;
+            yn = zmul({yp.x, yp.y}, t);
+        }
+        const dcx id = zinv(dn), yd = zmul(yn, id), term = zmul(yn, yd);
+        double2 G = a.G[s];
+        G.x += term.re;
+        G.y += term.im;
+        a.G[s] = G;
+        a.id[s] = make_double2(id.re, id.im);
+        a.y[s] = make_double2(yn.re, yn.im);
+        if (bn * zabs(yd) <= a.tol) a.frozen[s] = 1;
+        else running = 1;
+    }
+    running = __syncthreads_count(running);
+    if (threadIdx.x == 0) {
+        atomicAdd(a.counter + 1, (unsigned int)running);   // integer: order-independent
+        __threadfence();
+        if (atomicAdd(a.counter, 1u) == (unsigned int)a.n_blocks - 1) {
+            __threadfence();
+            const unsigned int cnt = atomicAdd(a.counter + 1, 0u);
+            a.counter[0] = 0u;
+            a.counter[1] = 0u;
+            *a.iter = a.j + 1;
+            if (cnt == 0 || bn == 0.0) *a.done = 4 * (a.j + 1) + 1;
+            else if (a.j + 1 >= a.max_iter) *a.done = 4 * (a.j + 1) + 2;
+        }
+    }
+}
+__global__ void __launch_bounds__(32) lz_shift_kernel(LzShiftArgs a) {
+    if (*a.done) return;
+    lz_shift_block(a, blockIdx.x);
+}
+
+// Bound by its random reads (a table entry and an amplitude per bond) and by
+// the FP64 pipe, so a bond costs four multiply-adds: its amplitude times the
+// conjugate character comes from a table in shared memory, and sqrt(o_r' / o_r'')
+// is 1 unless one of the two orbits is short. (With the quotient of the two
+// roots formed per bond and the sector index looked up behind the table the
+// 20-site product took 120 us, 4 dependent reads and about 20 FP64 operations
+// a bond.) The entries of kSecChunk bonds are read before their amplitudes, so
+// that the reads overlap.
+// SEC_DOT: the leading lz.n_blocks blocks carry out the shift recurrences of
+// the previous Lanczos iteration, which only the next check waits for.
+constexpr int kSecHvThreads = 128;
+constexpr int kSecChunk = 6;
 template <int EPI>
-__global__ void __launch_bounds__(kSecThreads) sec_hv_kernel(const SecHam h, SecHvArgs a) {
-    __shared__ double red[(kSecThreads / 32) * 3];
+__global__ void __launch_bounds__(kSecHvThreads) sec_hv_kernel(const __grid_constant__ SecHam h,
+                                                              const __grid_constant__ SecHvArgs a) {
+    __shared__ double red[(kSecHvThreads / 32) * 2];
+    __shared__ double2 tab[6 * kMaxGroup];   // amplitude times conj(chi)
+    if (EPI == SEC_DOT && a.done) {
+        const int d = *a.done;
+        if (d != 0 && d / 4 < a.iter) return;
+    }
+    const int nsb = EPI == SEC_DOT ? a.lz.n_blocks : 0;
+    if (EPI == SEC_DOT && (int)blockIdx.x < nsb) {
+        lz_shift_block(a.lz, blockIdx.x);
+        return;
+    }
+    for (int q = threadIdx.x; q < 6 * kMaxGroup; q += blockDim.x) {
+        const int g = q % kMaxGroup;
+        const double2 ch = g < a.ng ? a.chi[g] : make_double2(0.0, 0.0);
+        tab[q] = make_double2(h.c[q / kMaxGroup] * ch.x, -h.c[q / kMaxGroup] * ch.y);
+    }
+    __syncthreads();
+    const int blk = blockIdx.x - nsb, nblk = gridDim.x - nsb;
+    const uint32_t gmask = a.flag_full ? kLocFull - 1u : 31u;
     const double sc = a.in_scale ? *a.in_scale : 1.0;
-    double d0 = 0, d1 = 0, d2 = 0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.dim; i += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t r = a.orb_rep[a.sec_orbit[i]];
+    double d0 = 0, d1 = 0;
+    for (int64_t i = (int64_t)blk * blockDim.x + threadIdx.x; i < a.dim; i += (int64_t)nblk * blockDim.x) {
+        const uint32_t r = a.rep[i];
         const double so = a.sqo[i];
         const double2 v = a.in[i];
-        double diag = 0, ar = 0, ai = 0;
-        for (int b = 0; b < h.nb; ++b) {
-            const uint32_t m = h.mask[b];
-            const int par = (__popc(r & m) & 1) == 0;   // parallel spins
-            diag += par ? h.dg[b] : -h.dg[b];
-            const double c = par ? h.par[b] : h.anti[b];
-            if (c == 0.0) continue;
-            const uint32_t L = a.loc[r ^ m];
-            const int32_t j = a.sec_index[L >> 5];
-            if (j < 0) continue;
-            const double2 ch = a.chi[L & 31];
-            const double2 w = a.in[j];
-            const double f = c * so / a.sqo[j];
-            // conj(chi) w
-            ar += f * (ch.x * w.x + ch.y * w.y);
-            ai += f * (ch.x * w.y - ch.y * w.x);
+        const bool full = a.flag_full && so == a.full;
+        double ar = 0, ai = 0;
+        int anti[3] = {0, 0, 0};
+#pragma unroll
+        for (int g = 0; g < 3; ++g) {
+            for (int b = h.off[g]; b < h.off[g + 1]; b += kSecChunk) {
+                uint32_t L[kSecChunk];
+                double2 w[kSecChunk];
+                unsigned odd = 0;
+#pragma unroll
+                for (int u = 0; u < kSecChunk; ++u) {
+                    L[u] = kLocNone;
+                    if (b + u < h.off[g + 1]) {
+                        const uint32_t m = h.mask[b + u];
+                        const int o = __popc(r & m) & 1;   // antiparallel spins
+                        odd |= (unsigned)o << u;
+                        if (h.c[2 * g + o] != 0.0) L[u] = a.loc[r ^ m];
+                    }
+                }
+                anti[g] += __popc(odd);
+#pragma unroll
+                for (int u = 0; u < kSecChunk; ++u)
+                    if (L[u] != kLocNone) w[u] = a.in[L[u] >> 5];
+#pragma unroll
+                for (int u = 0; u < kSecChunk; ++u)
+                    if (L[u] != kLocNone) {
+                        double2 t = tab[(2 * g + ((odd >> u) & 1)) * kMaxGroup + (L[u] & gmask)];
+                        if (!full || !(L[u] & kLocFull)) {
+                            const double f = so / a.sqo[L[u] >> 5];
+                            t.x *= f;
+                            t.y *= f;
+                        }
+                        ar = fma(t.x, w[u].x, ar); ar = fma(-t.y, w[u].y, ar);
+                        ai = fma(t.x, w[u].y, ai); ai = fma(t.y, w[u].x, ai);
+                    }
+            }
         }
-        ar = (ar + diag * v.x) * sc;
-        ai = (ai + diag * v.y) * sc;
-        if (EPI == SEC_PLAIN) {
-            a.out[i] = make_double2(ar, ai);
-        } else if (EPI == SEC_TPQ) {
+        const double diag = (double)(h.off[2] - 2 * (anti[0] + anti[1])) * h.dgv[0] +
+                            (double)(h.off[3] - h.off[2] - 2 * anti[2]) * h.dgv[1];
+        ar = fma(diag, v.x, ar) * sc;
+        ai = fma(diag, v.y, ai) * sc;
+        if (EPI == SEC_TPQ) {
             const double vx = v.x * sc, vy = v.y * sc;
             const double ox = a.ell * vx - a.inv_n * ar, oy = a.ell * vy - a.inv_n * ai;
             a.out[i] = make_double2(ox, oy);
             d0 += vx * ar + vy * ai;
             d1 += ox * ox + oy * oy;
-            d2 += vx * vx + vy * vy;
         } else {
             a.out[i] = make_double2(ar, ai);
-            const double vx = v.x * sc, vy = v.y * sc;
-            d0 += vx * ar + vy * ai;
-            d2 += vx * vx + vy * vy;
+            if (EPI == SEC_DOT) d0 += sc * (v.x * ar + v.y * ai);
         }
     }
     if (EPI == SEC_PLAIN) return;
-    double v3[3] = {d0, d1, d2};
-    block_reduce<3>(v3, red);
-    if (threadIdx.x < 3) a.partials[(size_t)blockIdx.x * 3 + threadIdx.x] = red[threadIdx.x];
-    last_block_reduce<3>(a.partials, a.counter, a.result, red);
+    __shared__ double fin[2];
+    double v2[2] = {d0, d1};
+    block_reduce<2>(v2, red);
+    if (threadIdx.x < 2) a.partials[(size_t)blk * 2 + threadIdx.x] = red[threadIdx.x];
+    if (!last_block_reduce<2>(a.partials, a.counter, fin, red, nblk)) return;
+    if (threadIdx.x != 0) return;
+    if (EPI == SEC_DOT) {
+        *a.result = fin[0];
+    } else {
+        *a.stat_e = fin[0];
+        *a.stat_q2 = fin[1];
+        *a.next_scale = fin[1] > 0.0 ? 1.0 / sqrt(fin[1]) : 0.0;
+    }
 }
 
 // --------------------------------------------------------- Lanczos vectors
-// w = H q_j (in out, from SEC_DOT with a_j = <q_j|H q_j> in result[0]);
-// w <- w - a_j q_j - b_j q_{j-1}, |w|^2 -> result; b_j from *beta_cur
+// With q_j = s_j Q_j (s_j = 1 / b_j, Q_j unnormalised) and w = H q_j in W:
+// W <- W - a_j q_j - b_j q_{j-1} = Q_{j+1}, b_{j+1} = |W|, s_{j+1} = 1 / b_{j+1}
 struct LzArgs {
     int64_t dim;
     double2 *w;
     const double2 *q, *qp;
-    const double *alpha;      // device a_j (the SEC_DOT result)
-    const double *beta;       // device b_j (0 at j = 0)
+    const double *alpha;                 // a_j
+    const double *beta;                  // b_j (0 at j = 0)
+    const double *s, *sp;                // s_j, s_{j-1}
+    double *beta_next, *s_next;          // b_{j+1}, s_{j+1}
     double *partials;
     unsigned int *counter;
-    double *result;           // [1]: |w|^2
     const int *done;
 };
 
 __global__ void __launch_bounds__(kSecThreads) lz_update_kernel(LzArgs a) {
     __shared__ double red[kSecThreads / 32];
+    __shared__ double fin[1];
     if (*a.done) return;
-    const double al = *a.alpha, be = *a.beta;
+    const double al = *a.alpha * *a.s, be = *a.beta * *a.sp;
     double n2 = 0;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.dim; i += (int64_t)gridDim.x * blockDim.x) {
         double2 w = a.w[i];
@@ -290,76 +449,11 @@ __global__ void __launch_bounds__(kSecThreads) lz_update_kernel(LzArgs a) {
     double v[1] = {n2};
     block_reduce<1>(v, red);
     if (threadIdx.x == 0) a.partials[blockIdx.x] = red[0];
-    last_block_reduce<1>(a.partials, a.counter, a.result, red);
-}
-
-// q_{j+1} = w / b_{j+1} (in place of q_{j-1})
-__global__ void lz_scale_kernel(int64_t dim, const double2 *w, double2 *qn, const double *beta_next, const int *done) {
-    if (*done) return;
-    const double b = *beta_next;
-    const double s = b > 0 ? 1.0 / b : 0.0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < dim; i += (int64_t)gridDim.x * blockDim.x) {
-        const double2 x = w[i];
-        qn[i] = make_double2(x.x * s, x.y * s);
-    }
-}
-
-// scalars of iteration j: a_j (alpha), b_{j+1} = sqrt(|w|^2); per shift the
-// pivot d_j, y_j, G, frozen once |b_{j+1} y_j / d_j| <= tol; done when every
-// shift is frozen, b_{j+1} vanished, or j + 1 = max_iter
-struct LzShiftArgs {
-    int n_shift, max_iter;
-    double tol;
-    const double2 *z;          // [n_shift]
-    const double *alpha;       // a_j
-    double *beta;              // [2]: b_j (read), b_{j+1} (written from w2)
-    const double *w2;          // |w|^2
-    double2 *d, *y, *G;        // [n_shift]
-    int *frozen;               // [n_shift]
-    int *iter;                 // j
-    int *done;
-    int *active_count;         // scratch: shifts still running after this iteration
-};
-
-__global__ void __launch_bounds__(256) lz_shift_kernel(LzShiftArgs a) {
-    if (*a.done) return;
-    const int j = *a.iter;
-    const double al = *a.alpha, bj = a.beta[0];
-    const double bn = sqrt(fmax(*a.w2, 0.0));
-    __shared__ int cnt;
-    if (threadIdx.x == 0) cnt = 0;
-    __syncthreads();
-    int mine = 0;
-    for (int s = threadIdx.x; s < a.n_shift; s += blockDim.x) {
-        if (a.frozen[s]) continue;
-        const double2 z = a.z[s];
-        dcx dn, yn;
-        if (j == 0) {
-            dn = {z.x - al, z.y};
-            yn = {1.0, 0.0};
-        } else {
-            const double2 dp = a.d[s], yp = a.y[s];
-            const dcx t = zdiv({bj * bj, 0.0}, {dp.x, dp.y});
-            dn = {z.x - al - t.re, z.y - t.im};
-            yn = zmul({yp.x, yp.y}, zdiv({bj, 0.0}, {dp.x, dp.y}));
-        }
-        const dcx term = zdiv(zmul(yn, yn), dn);
-        double2 G = a.G[s];
-        G.x += term.re;
-        G.y += term.im;
-        a.G[s] = G;
-        a.d[s] = make_double2(dn.re, dn.im);
-        a.y[s] = make_double2(yn.re, yn.im);
-        const double res = bn * zabs(zdiv(yn, dn));
-        if (res <= a.tol) a.frozen[s] = 1;
-        else ++mine;
-    }
-    atomicAdd(&cnt, mine);
-    __syncthreads();
+    if (!last_block_reduce<1>(a.partials, a.counter, fin, red)) return;
     if (threadIdx.x == 0) {
-        a.beta[0] = bn;   // b_{j+1} becomes b_j of the next iteration
-        *a.iter = j + 1;
-        if (cnt == 0 || bn == 0.0 || j + 1 >= a.max_iter) *a.done = (cnt == 0 || bn == 0.0) ? 1 : 2;
+        const double b = sqrt(fin[0]);
+        *a.beta_next = b;
+        *a.s_next = b > 0.0 ? 1.0 / b : 0.0;
     }
 }
 
@@ -455,10 +549,11 @@ struct ftk_sector {
     uint32_t *orb_rep = nullptr, *orb_stab = nullptr;   // [n_orb]
     int32_t *sec_index = nullptr;        // [n_orb]
     int32_t *sec_orbit = nullptr;        // [dim]
+    uint32_t *sec_rep = nullptr;         // [dim]
     double *sqo = nullptr;               // [dim]
     double2 *dchi = nullptr;             // [ng]
     double2 *vec = nullptr;              // [n_slots][dim]
-    double *scal = nullptr;              // scalars / reductions: [0..63] results, then partials
+    double *scal = nullptr;              // scalars [0..63], statistics of kStatCap steps, partials
     unsigned int *counter = nullptr;
     int *iflag = nullptr;                // [8]: done, iter, ...
     SecHam sh{};
@@ -486,6 +581,10 @@ ftk_status sfail(ftk_sector *s, ftk_status st, const std::string &m) {
     } while (0)
 
 constexpr int kPartialCap = 8192;   // reduction partials (grid cap)
+constexpr int kStatCap = 1024;      // mTPQ steps between reads of their statistics
+// scal: [8..9] scale of the state of an even / odd step; Lanczos rings of four
+enum { SC_DOT = 0, SC_NORM = 1, SC_SCALE = 8, SC_ALPHA = 16, SC_BETA = 20, SC_INV = 24, SC_STAT = 64,
+       SC_PART = SC_STAT + 2 * kStatCap };
 
 double2 *slot_ptr(ftk_sector *s, int k) { return s->vec + (size_t)k * s->dim; }
 
@@ -504,22 +603,41 @@ SecGroup group_args(ftk_sector *s) {
     return g;
 }
 
+int hv_grid(ftk_sector *s) {
+    const int64_t want = (s->dim + kSecHvThreads - 1) / kSecHvThreads;
+    return (int)std::max<int64_t>(1, std::min<int64_t>(want, std::min<int64_t>(kPartialCap, 16LL * s->ham.n_sm)));
+}
+
 SecHvArgs hv_args(ftk_sector *s, const double2 *in, double2 *out) {
     SecHvArgs a{};
     a.dim = s->dim;
     a.loc = s->loc;
-    a.orb_rep = s->orb_rep;
-    a.sec_index = s->sec_index;
-    a.sec_orbit = s->sec_orbit;
+    a.rep = s->sec_rep;
     a.sqo = s->sqo;
+    a.full = std::sqrt((double)s->ng);
+    a.flag_full = s->ng <= (int)kLocFull;
+    a.ng = s->ng;
     a.chi = s->dchi;
     a.in = in;
     a.out = out;
     a.inv_n = 1.0 / s->n;
-    a.partials = s->scal + 64;
+    a.partials = s->scal + SC_PART;
     a.counter = s->counter;
-    a.result = s->scal;
+    a.result = s->scal + SC_DOT;
     return a;
+}
+
+// |v|^2 of a sector vector to *n2 (synchronises)
+ftk_status sec_norm2(ftk_sector *sec, const double2 *v, double *n2) {
+    InitArgs ia{};
+    ia.dim = (uint64_t)sec->dim;
+    ia.partials = sec->scal + SC_PART;
+    ia.counter = sec->counter;
+    ia.result = sec->scal + SC_NORM;
+    SLAUNCH(launch_norm(FTK_FP64, v, ia, sec_grid(sec, sec->dim), sec->ham.stream));
+    SCK(cudaMemcpyAsync(n2, sec->scal + SC_NORM, sizeof(double), cudaMemcpyDeviceToHost, sec->ham.stream));
+    SCK(cudaStreamSynchronize(sec->ham.stream));
+    return FTK_OK;
 }
 
 }  // namespace
@@ -600,17 +718,17 @@ ftk_status ftk_sector_create(ftk_ctx *ctx, const int32_t *perms, int32_t n_g, co
     for (int a = 0; a < n_g; ++a)
         for (int b = 0; b < n_g; ++b)
             if (mul[(size_t)a * n_g + b] == 0) sec->ginv[a] = b;
-    // bonds
-    sec->sh.nb = h.nb;
-    for (int q = 0; q < h.nb; ++q) {
-        const int i = h.bonds[3 * q], j = h.bonds[3 * q + 1], g = h.bonds[3 * q + 2];
-        sec->sh.mask[q] = (1u << i) | (1u << j);
-        double pa = 0, an = 0;
-        bond_coefficients(g, h.K, h.J, &pa, &an);
-        sec->sh.par[q] = pa;
-        sec->sh.anti[q] = an;
-        sec->sh.dg[q] = g == 2 ? (h.J + h.K) / 4 : h.J / 4;
+    // bonds, sorted by type
+    int nbs = 0;
+    for (int g = 0; g < 3; ++g) {
+        sec->sh.off[g] = nbs;
+        for (int q = 0; q < h.nb; ++q)
+            if (h.bonds[3 * q + 2] == g) sec->sh.mask[nbs++] = (1u << h.bonds[3 * q]) | (1u << h.bonds[3 * q + 1]);
+        bond_coefficients(g, h.K, h.J, &sec->sh.c[2 * g], &sec->sh.c[2 * g + 1]);
     }
+    sec->sh.off[3] = nbs;
+    sec->sh.dgv[0] = h.J / 4;
+    sec->sh.dgv[1] = (h.J + h.K) / 4;
     // byte tables: image of byte value v at byte position p under g
     std::vector<uint32_t> tab((size_t)n_g * sec->nbytes * 256, 0);
     for (int g = 0; g < n_g; ++g)
@@ -673,8 +791,6 @@ ftk_status ftk_sector_create(ftk_ctx *ctx, const int32_t *perms, int32_t n_g, co
     CK2(cudaMalloc(&sec->orb_stab, 4 * (size_t)tot));
     sec_compact_kernel<<<n_blocks, kSecThreads, tab_bytes, st>>>(G, D, rep_of, counts, sec->orb_rep, sec->orb_stab, idx_of);
     CK2(cudaGetLastError());
-    sec_loc_kernel<<<ggrid, kSecThreads, 0, st>>>(D, rep_of, g_of, idx_of, sec->loc);
-    CK2(cudaGetLastError());
     // sector basis
     CK2(cudaMalloc(&sec->dchi, sizeof(double2) * n_g));
     CK2(cudaMemcpyAsync(sec->dchi, chi, sizeof(double2) * n_g, cudaMemcpyHostToDevice, st));
@@ -693,12 +809,16 @@ ftk_status ftk_sector_create(ftk_ctx *ctx, const int32_t *perms, int32_t n_g, co
     CK2(cudaMalloc(&sec->sec_index, sizeof(int32_t) * tot));
     CK2(cudaMalloc(&sec->sec_orbit, sizeof(int32_t) * dim));
     CK2(cudaMalloc(&sec->sqo, sizeof(double) * dim));
-    sec_fill_kernel<<<sec_grid(sec, tot), kSecThreads, 0, st>>>((int)tot, n_g, sec->orb_stab, flag, fpos, sec->sec_index,
-                                                                 sec->sec_orbit, sec->sqo);
+    CK2(cudaMalloc(&sec->sec_rep, sizeof(uint32_t) * dim));
+    sec_fill_kernel<<<sec_grid(sec, tot), kSecThreads, 0, st>>>((int)tot, n_g, sec->orb_rep, sec->orb_stab, flag, fpos,
+                                                                sec->sec_index, sec->sec_orbit, sec->sec_rep, sec->sqo);
+    CK2(cudaGetLastError());
+    sec_loc_kernel<<<ggrid, kSecThreads, 0, st>>>(D, rep_of, g_of, idx_of, sec->sec_index, sec->orb_stab,
+                                                  n_g <= (int)kLocFull, sec->loc);
     CK2(cudaGetLastError());
     CK2(cudaMalloc(&sec->vec, sizeof(double2) * (size_t)dim * n_slots));
     CK2(cudaMemsetAsync(sec->vec, 0, sizeof(double2) * (size_t)dim * n_slots, st));
-    CK2(cudaMalloc(&sec->scal, sizeof(double) * (64 + 3 * kPartialCap)));
+    CK2(cudaMalloc(&sec->scal, sizeof(double) * (SC_PART + 3 * kPartialCap)));
     CK2(cudaMemsetAsync(sec->scal, 0, sizeof(double) * 64, st));
     CK2(cudaMalloc(&sec->counter, sizeof(unsigned int) * 4));
     CK2(cudaMemsetAsync(sec->counter, 0, sizeof(unsigned int) * 4, st));
@@ -717,7 +837,7 @@ void ftk_sector_destroy(ftk_sector *s) {
     if (!s) return;
     if (s->ham.stream) cudaStreamSynchronize(s->ham.stream);
     cudaFree(s->tab); cudaFree(s->loc); cudaFree(s->orb_rep); cudaFree(s->orb_stab); cudaFree(s->sec_index);
-    cudaFree(s->sec_orbit); cudaFree(s->sqo); cudaFree(s->dchi); cudaFree(s->vec); cudaFree(s->scal);
+    cudaFree(s->sec_orbit); cudaFree(s->sec_rep); cudaFree(s->sqo); cudaFree(s->dchi); cudaFree(s->vec); cudaFree(s->scal);
     cudaFree(s->counter); cudaFree(s->iflag);
     delete s;
 }
@@ -785,7 +905,7 @@ ftk_status ftk_sector_hv(ftk_sector *sec, int32_t slot_in, int32_t slot_out) {
     if (!sec || slot_in < 0 || slot_out < 0 || slot_in >= sec->n_slots || slot_out >= sec->n_slots || slot_in == slot_out)
         return sfail(sec, FTK_EINVAL, "ftk_sector_hv: bad slots");
     SecHvArgs a = hv_args(sec, slot_ptr(sec, slot_in), slot_ptr(sec, slot_out));
-    sec_hv_kernel<SEC_PLAIN><<<sec_grid(sec, sec->dim), kSecThreads, 0, sec->ham.stream>>>(sec->sh, a);
+    sec_hv_kernel<SEC_PLAIN><<<hv_grid(sec), kSecHvThreads, 0, sec->ham.stream>>>(sec->sh, a);
     SCK(cudaGetLastError());
     ++*sec->ham.launches;
     return FTK_OK;
@@ -806,53 +926,58 @@ ftk_status ftk_sector_tpq(ftk_sector *sec, int32_t slot_state, int32_t slot_work
         if (first_save_slot + k == slot_state || first_save_slot + k == slot_work)
             return sfail(sec, FTK_EINVAL, "ftk_sector_tpq: save slots overlap the state or work slot");
     cudaStream_t st = sec->ham.stream;
-    // normalise the initial state (its norm is returned: the sector's share of
-    // a projected state)
-    {
-        SecHvArgs a = hv_args(sec, slot_ptr(sec, slot_state), slot_ptr(sec, slot_work));
-        sec_hv_kernel<SEC_DOT><<<sec_grid(sec, sec->dim), kSecThreads, 0, st>>>(sec->sh, a);
-        SCK(cudaGetLastError());
-        ++*sec->ham.launches;
-        double r[3];
-        SCK(cudaMemcpyAsync(r, sec->scal, sizeof r, cudaMemcpyDeviceToHost, st));
-        SCK(cudaStreamSynchronize(st));
-        if (!(r[2] > 0)) return sfail(sec, FTK_EINVAL, "ftk_sector_tpq: the state has no component in this sector");
-        if (lognorm0_out) *lognorm0_out = 0.5 * std::log(r[2]);
-        const double sc = 1.0 / std::sqrt(r[2]);
-        SCK(cudaMemcpyAsync(sec->scal + 8, &sc, sizeof sc, cudaMemcpyHostToDevice, st));
-        sec_scale_kernel<<<sec_grid(sec, sec->dim), kSecThreads, 0, st>>>(sec->dim, slot_ptr(sec, slot_state),
-                                                                           slot_ptr(sec, slot_state), sec->scal + 8);
-        SCK(cudaGetLastError());
-        ++*sec->ham.launches;
-    }
+    // the initial state's norm is returned (the sector's share of a projected
+    // state); every state is kept with its scale, the two slots in turn, and
+    // the statistics stay on the device for kStatCap steps
+    double n2 = 0;
+    ftk_status ns = sec_norm2(sec, slot_ptr(sec, slot_state), &n2);
+    if (ns) return ns;
+    if (!(n2 > 0)) return sfail(sec, FTK_EINVAL, "ftk_sector_tpq: the state has no component in this sector");
+    if (lognorm0_out) *lognorm0_out = 0.5 * std::log(n2);
+    double *scale = sec->scal + SC_SCALE, *stat = sec->scal + SC_STAT;
+    const double sc = 1.0 / std::sqrt(n2);
+    SCK(cudaMemcpyAsync(scale, &sc, sizeof sc, cudaMemcpyHostToDevice, st));
+    double2 *buf[2] = {slot_ptr(sec, slot_state), slot_ptr(sec, slot_work)};
     double logq = 0.0;
     int saved = 0;
-    for (int k = 0; k < n_steps; ++k) {
-        double2 *cur = slot_ptr(sec, slot_state), *wk = slot_ptr(sec, slot_work);
-        if (k % save_every == 0) {
-            SCK(cudaMemcpyAsync(slot_ptr(sec, first_save_slot + saved), cur, sizeof(double2) * sec->dim,
-                                cudaMemcpyDeviceToDevice, st));
-            ++saved;
+    std::vector<double> host(2 * (size_t)std::min(std::max(n_steps, 1), kStatCap));
+    for (int k0 = 0; k0 < n_steps; k0 += kStatCap) {
+        const int nk = std::min(kStatCap, n_steps - k0);
+        for (int k = k0; k < k0 + nk; ++k) {
+            double2 *cur = buf[k & 1], *nxt = buf[(k + 1) & 1];
+            if (k % save_every == 0) {
+                sec_scale_kernel<<<sec_grid(sec, sec->dim), kSecThreads, 0, st>>>(
+                    sec->dim, cur, slot_ptr(sec, first_save_slot + saved), scale + (k & 1));
+                SCK(cudaGetLastError());
+                ++*sec->ham.launches;
+                ++saved;
+            }
+            SecHvArgs a = hv_args(sec, cur, nxt);
+            a.ell = ell;
+            a.in_scale = scale + (k & 1);
+            a.next_scale = scale + ((k + 1) & 1);
+            a.stat_e = stat + (k - k0);
+            a.stat_q2 = stat + kStatCap + (k - k0);
+            sec_hv_kernel<SEC_TPQ><<<hv_grid(sec), kSecHvThreads, 0, st>>>(sec->sh, a);
+            SCK(cudaGetLastError());
+            ++*sec->ham.launches;
         }
-        SecHvArgs a = hv_args(sec, cur, wk);
-        a.ell = ell;
-        sec_hv_kernel<SEC_TPQ><<<sec_grid(sec, sec->dim), kSecThreads, 0, st>>>(sec->sh, a);
-        SCK(cudaGetLastError());
-        ++*sec->ham.launches;
-        double r[3];
-        SCK(cudaMemcpyAsync(r, sec->scal, sizeof r, cudaMemcpyDeviceToHost, st));
+        SCK(cudaMemcpyAsync(host.data(), stat, sizeof(double) * nk, cudaMemcpyDeviceToHost, st));
+        SCK(cudaMemcpyAsync(host.data() + nk, stat + kStatCap, sizeof(double) * nk, cudaMemcpyDeviceToHost, st));
         SCK(cudaStreamSynchronize(st));
         // u_k = <psi_k|H|psi_k> / N (psi_k normalised); log Q_k; q_k = |psi'|
-        if (u_out) u_out[k] = r[0] / sec->n;
-        if (logq_out) logq_out[k] = logq;
-        if (!(r[1] > 0)) return sfail(sec, FTK_EBREAKDOWN, "ftk_sector_tpq: the state vanished");
-        logq += 0.5 * std::log(r[1]);
-        const double sc = 1.0 / std::sqrt(r[1]);
-        SCK(cudaMemcpyAsync(sec->scal + 8, &sc, sizeof sc, cudaMemcpyHostToDevice, st));
-        sec_scale_kernel<<<sec_grid(sec, sec->dim), kSecThreads, 0, st>>>(sec->dim, wk, cur, sec->scal + 8);
-        SCK(cudaGetLastError());
-        ++*sec->ham.launches;
+        for (int k = 0; k < nk; ++k) {
+            if (u_out) u_out[k0 + k] = host[k] / sec->n;
+            if (logq_out) logq_out[k0 + k] = logq;
+            if (!(host[nk + k] > 0)) return sfail(sec, FTK_EBREAKDOWN, "ftk_sector_tpq: the state vanished");
+            logq += 0.5 * std::log(host[nk + k]);
+        }
     }
+    // the last state, normalised, into its slot
+    sec_scale_kernel<<<sec_grid(sec, sec->dim), kSecThreads, 0, st>>>(sec->dim, buf[n_steps & 1], buf[0],
+                                                                       scale + (n_steps & 1));
+    SCK(cudaGetLastError());
+    ++*sec->ham.launches;
     SCK(cudaStreamSynchronize(st));
     return FTK_OK;
 }
@@ -903,29 +1028,22 @@ ftk_status ftk_sector_green(ftk_sector *sec, int32_t slot, const double *shifts,
     cudaStream_t st = sec->ham.stream;
     // vectors: q_prev, q, w in the three slots after `slot` (cyclic)
     const int s1 = (slot + 1) % sec->n_slots, s2 = (slot + 2) % sec->n_slots, s3 = (slot + 3) % sec->n_slots;
-    double2 *lam = slot_ptr(sec, slot), *qa = slot_ptr(sec, s1), *qb = slot_ptr(sec, s2), *w = slot_ptr(sec, s3);
-    // |lambda|^2 and q_0 = lambda / |lambda|, q_{-1} = 0
-    SecHvArgs a0 = hv_args(sec, lam, w);
-    sec_hv_kernel<SEC_DOT><<<sec_grid(sec, sec->dim), kSecThreads, 0, st>>>(sec->sh, a0);
-    SCK(cudaGetLastError());
-    double r[3];
-    SCK(cudaMemcpyAsync(r, sec->scal, sizeof r, cudaMemcpyDeviceToHost, st));
-    SCK(cudaStreamSynchronize(st));
-    const double lam2 = r[2];
+    double2 *lam = slot_ptr(sec, slot), *buf[3] = {slot_ptr(sec, s1), slot_ptr(sec, s2), slot_ptr(sec, s3)};
+    // Q_0 = lambda, s_0 = 1 / |lambda|; Q_1, Q_2, ... in the three slots in turn
+    double lam2 = 0;
+    ftk_status ns = sec_norm2(sec, lam, &lam2);
+    if (ns) return ns;
     if (!(lam2 > 0)) {   // a zero probe: G = 0
         std::fill(G_out, G_out + 2 * (size_t)n_shift, 0.0);
         if (iters_out) *iters_out = 0;
         return FTK_OK;
     }
     const double sc = 1.0 / std::sqrt(lam2);
-    // device scalars (scal): [0..2] dot results, [8] scale, [16] alpha, [17..18] beta, [20] |w|^2
-    SCK(cudaMemcpyAsync(sec->scal + 8, &sc, sizeof sc, cudaMemcpyHostToDevice, st));
-    sec_scale_kernel<<<sec_grid(sec, sec->dim), kSecThreads, 0, st>>>(sec->dim, lam, qb, sec->scal + 8);
-    SCK(cudaGetLastError());
-    SCK(cudaMemsetAsync(qa, 0, sizeof(double2) * sec->dim, st));
-    SCK(cudaMemsetAsync(sec->scal + 17, 0, sizeof(double) * 2, st));
+    double *alpha = sec->scal + SC_ALPHA, *beta = sec->scal + SC_BETA, *inv = sec->scal + SC_INV;
+    SCK(cudaMemsetAsync(alpha, 0, sizeof(double) * 12, st));   // the three rings; b_0 = 0, s_{-1} = 0
+    SCK(cudaMemcpyAsync(inv, &sc, sizeof sc, cudaMemcpyHostToDevice, st));
     SCK(cudaMemsetAsync(sec->iflag, 0, sizeof(int) * 8, st));
-    // per-shift state in a scratch allocation: z, d, y, G, frozen
+    // per-shift state in a scratch allocation: z, 1/d, y, G, frozen
     double2 *zd = nullptr;
     SCK(cudaMalloc(&zd, sizeof(double2) * 4 * n_shift + sizeof(int) * n_shift));
     double2 *dz = zd, *dd = zd + n_shift, *dy = zd + 2 * n_shift, *dG = zd + 3 * n_shift;
@@ -935,48 +1053,65 @@ ftk_status ftk_sector_green(ftk_sector *sec, int32_t slot, const double *shifts,
     if (e != cudaSuccess) { cudaFree(zd); return sfail(sec, FTK_ECUDA, cudaGetErrorString(e)); }
     LzShiftArgs la{};
     la.n_shift = n_shift;
+    la.n_blocks = (n_shift + kShiftsPerBlock - 1) / kShiftsPerBlock;
     la.max_iter = max_iter;
     la.tol = tol;
     la.z = dz;
-    la.alpha = sec->scal;          // SEC_DOT result[0] = <q|Hq> (q normalised, real part)
-    la.beta = sec->scal + 17;
-    la.w2 = sec->scal + 20;
-    la.d = dd;
+    la.id = dd;
     la.y = dy;
     la.G = dG;
     la.frozen = dfz;
     la.iter = sec->iflag + 1;
     la.done = sec->iflag;
+    la.counter = sec->counter + 2;
+    auto shift_args = [&](int j) {
+        LzShiftArgs a = la;
+        a.j = j;
+        a.alpha = alpha + (j & 3);
+        a.beta = beta + (j & 3);
+        a.beta_next = beta + ((j + 1) & 3);
+        return a;
+    };
     int done = 0, it = 0;
-    double2 *qp = qa, *qc = qb;    // q_{j-1}, q_j
     while (e == cudaSuccess) {
         for (int c = 0; c < 32 && it < max_iter; ++c, ++it) {
-            // w = H q_j, a_j = <q_j|H q_j>; skipped once done (the dot kernel
-            // itself runs, its result is unused)
-            SecHvArgs a = hv_args(sec, qc, w);
-            sec_hv_kernel<SEC_DOT><<<sec_grid(sec, sec->dim), kSecThreads, 0, st>>>(sec->sh, a);
+            // w = H q_j, a_j = <q_j|H q_j>, with the shifts of iteration j - 1
+            const double2 *Q = it == 0 ? lam : buf[(it - 1) % 3];
+            const double2 *P = it < 2 ? lam : buf[(it - 2) % 3];   // b_0 = 0: unused at j = 0
+            double2 *w = buf[it % 3];
+            SecHvArgs a = hv_args(sec, Q, w);
+            a.in_scale = inv + (it & 3);
+            a.result = alpha + (it & 3);
+            a.done = sec->iflag;
+            a.iter = it;
+            if (it > 0) a.lz = shift_args(it - 1);
+            sec_hv_kernel<SEC_DOT><<<hv_grid(sec) + a.lz.n_blocks, kSecHvThreads, 0, st>>>(sec->sh, a);
             LzArgs u{};
             u.dim = sec->dim;
             u.w = w;
-            u.q = qc;
-            u.qp = qp;
-            u.alpha = sec->scal;
-            u.beta = sec->scal + 17;
-            u.partials = sec->scal + 64;
+            u.q = Q;
+            u.qp = P;
+            u.alpha = alpha + (it & 3);
+            u.beta = beta + (it & 3);
+            u.s = inv + (it & 3);
+            u.sp = inv + ((it + 3) & 3);
+            u.beta_next = beta + ((it + 1) & 3);
+            u.s_next = inv + ((it + 1) & 3);
+            u.partials = sec->scal + SC_PART;
             u.counter = sec->counter + 1;
-            u.result = sec->scal + 20;
             u.done = sec->iflag;
             lz_update_kernel<<<sec_grid(sec, sec->dim), kSecThreads, 0, st>>>(u);
-            lz_shift_kernel<<<1, 256, 0, st>>>(la);
-            // q_{j+1} = w / b_{j+1} into q_{j-1}'s buffer
-            lz_scale_kernel<<<sec_grid(sec, sec->dim), kSecThreads, 0, st>>>(sec->dim, w, qp, sec->scal + 17, sec->iflag);
             e = cudaGetLastError();
             if (e != cudaSuccess) break;
-            *sec->ham.launches += 4;
-            std::swap(qp, qc);
+            *sec->ham.launches += 2;
         }
         if (e != cudaSuccess) break;
-        e = cudaMemcpyAsync(&done, sec->iflag, sizeof(int), cudaMemcpyDeviceToHost, st);
+        if (it >= max_iter) {   // the shifts of the last iteration
+            lz_shift_kernel<<<la.n_blocks, 32, 0, st>>>(shift_args(it - 1));
+            e = cudaGetLastError();
+            ++*sec->ham.launches;
+        }
+        if (e == cudaSuccess) e = cudaMemcpyAsync(&done, sec->iflag, sizeof(int), cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         if (done || it >= max_iter) break;
     }
@@ -990,7 +1125,7 @@ ftk_status ftk_sector_green(ftk_sector *sec, int32_t slot, const double *shifts,
     if (e != cudaSuccess) return sfail(sec, FTK_ECUDA, cudaGetErrorString(e));
     for (size_t i = 0; i < G.size(); ++i) G_out[i] = lam2 * G[i];
     if (iters_out) *iters_out = iters;
-    if (done != 1) return sfail(sec, FTK_ENOCONV, "ftk_sector_green: max_iter reached");
+    if (done % 4 != 1) return sfail(sec, FTK_ENOCONV, "ftk_sector_green: max_iter reached");
     return FTK_OK;
 }
 
