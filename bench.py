@@ -356,7 +356,7 @@ def run_gpu(args):
                    else None)
         roof = {"bound": "hbm", "achieved": round(alg / t_hv / 1e9, 2), "peak": peak, "unit": "GB/s",
                 "frac": round(alg / t_hv / 1e9 / peak, 4), "traffic": traffic, "peak_kind": peak_kind,
-                "kernel": f"hv_pass_df_kernel (double-float H.v, {n_rhs} columns, one per launch; tile "
+                "kernel": f"hv_df_kernel (double-float H.v, {n_rhs} columns; tile "
                           f"2^{tile_bits}, {n_pass} passes)",
                 "bytes_per_launch_set": alg, "hv_us": round(t_hv * 1e6, 2),
                 "alu": {"achieved": round(ops / t_hv / 1e12, 3), "peak": round(alu_peak, 2),
@@ -376,8 +376,9 @@ def run_gpu(args):
     t_hv1 = time_hv(ctx1, torch, 1, torch.complex64)
     p1 = ctx1.plan_info()
     ctx1.close()
-    # the FP64 H.v (mTPQ and the plain FP64 solve) against the FP64 pipe:
-    # 2 DFMA (4 flops) per amplitude and term (bonds + diagonal)
+    # the FP64 H.v (mTPQ and the plain FP64 solve) against the FP64 pipe, in
+    # equivalent flops: 2 DFMA (4 flops) per amplitude and term (bonds +
+    # diagonal); the sums run in 64-bit integers, so the figure may exceed 1
     ctx2 = ftk.Context(cl, K_COUPLING, J_COUPLING, "fp64", max_rhs=1)
     t_hv64 = time_hv(ctx2, torch, 1, torch.complex128)
     p64 = ctx2.plan_info()
@@ -410,7 +411,7 @@ def run_gpu(args):
     roof["hv_fp32_by_n"] = by_n
 
     # the batched configuration's knob: FP64 blocked H.V time per column
-    # against the block width (tile size and column chunk autotuned per width)
+    # against the block width (plan autotuned per width)
     blocked = {"B": [], "us_per_column": [], "plan": []}
     if not args.no_block_sweep:
         for B in (1, 4, 8, 16, 32):

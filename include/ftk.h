@@ -393,7 +393,8 @@ ftk_status ftk_hv(ftk_ctx *ctx, const void *v_dev, void *out_dev, int32_t n_rhs)
  * -1 - j probe slot j. Synchronises. */
 ftk_status ftk_get_vector(ftk_ctx *ctx, int32_t which, double *host_out);
 
-/* Number of H.v passes the plan uses, and the tile bits. */
+/* Number of H.v passes the plan uses, and the tile bits (1 and n_sites for a
+ * small vector, whose product is one launch without tiles). */
 ftk_status ftk_plan_info(const ftk_ctx *ctx, int32_t *n_passes, int32_t *tile_bits);
 
 /* Site relabelling that lets H.v run in fewer tiled passes (the layout
@@ -425,12 +426,13 @@ ftk_status ftk_set_relax(ftk_ctx *ctx, double theta);
 
 /* Autotuner of the blocked H.V (the batching knob of the Sec. IV.A product
  * on this hardware). Times, on scratch vectors in the context's Krylov
- * region, every admissible plan for n_rhs right-hand sides: column chunk
- * width (1, 2, 4 or 8 vectors per launch) x tile size (the two to three
- * largest tiles that fit), and installs the fastest one for later ftk_hv,
+ * region, every admissible plan for n_rhs right-hand sides: the two to three
+ * largest tiles that fit and, for small vectors, the product in one launch
+ * without tiles, and installs the fastest one for later ftk_hv,
  * ftk_shifted_cocg (which = 0, the context's matvec precision) or
  * ftk_tpq_step (which = 1, FP64, n_rhs = 1) calls. Outputs (may be NULL):
- * the chosen tile bits and chunk width and its time per H.V in us.
+ * the chosen tile bits (n_sites without tiles), the vectors a CTA takes (1 for
+ * tiles, n_rhs without) and its time per H.V in us.
  * n_rhs: a power of two <= max_rhs. Overwrites the Krylov region (call it
  * outside a solve). Synchronises. */
 ftk_status ftk_autotune(ftk_ctx *ctx, int32_t n_rhs, int32_t which, int32_t *tile_bits_out, int32_t *cols_out,

@@ -64,6 +64,7 @@ struct Small {
     unsigned int counters[8];
     unsigned int upd_counters[FTK_MAX_RHS];  // tickets of the updates' reductions, per column
     unsigned int hv_counters[FTK_MAX_RHS];   // tickets of the products' reductions, per column
+    FixRange range[FTK_MAX_RHS];             // exponents of the FP64 products' inputs
     double hv_dots[FTK_MAX_RHS * FTK_HV_DOTS];
     double upd_dots[FTK_MAX_RHS * FTK_UPD_DOTS];
     double op_dots[4];
@@ -74,10 +75,13 @@ struct Small {
 };
 
 struct Plan {
-    int tile_bits = 0, chunk_bits = 0, threads = 512, grid = 0;
-    size_t smem = 0;
-    bool gather = false;             // one launch over the whole vector (ftk_gather.cu), no passes
+    int tile_bits = 0, chunk_bits = 0, grid = 0;
+    bool fix = false;                // FP64: the passes have a fixed-point form
+    // one launch per element where not empty: the whole vector (no passes), or
+    // the passes of tiles too small for the tiled kernels
+    std::vector<GatherDesc> gathers;
     std::vector<PassDesc> passes;
+    int n_passes() const { return (int)(gathers.empty() ? passes.size() : gathers.size()); }
 };
 
 }  // namespace
@@ -154,53 +158,49 @@ void ftk::set_thread_error(const char *msg) { g_create_err = msg; }
 
 namespace {
 
-// Plan the passes of H.V for column chunks of bc right-hand sides: the
-// planner with its local search first; if that plan cannot be laid out for
-// the kernel (or needs too much shared memory), the greedy plan alone.
-bool plan_passes_with(ftk_ctx *ctx, int prec, int bc, int tile_bits, long local_steps, Plan &pl) {
+// Plan the passes of H.V: the planner with its local search, laid out for the
+// tiled kernels or, for tiles too small for them, as gather launches.
+bool plan_passes(ftk_ctx *ctx, int prec, int tile_bits, Plan &pl, long local_steps = kPlanLocalSteps) {
     PlanBond pb[2 * FTK_MAX_PASS_BONDS];
     for (int q = 0; q < ctx->nb; ++q) pb[q] = {ctx->bonds[q].i, ctx->bonds[q].j, ctx->bonds[q].g};
     PassDesc pd[FTK_MAX_PASSES];
-    const int np = plan_hv_passes(ctx->n, pb, ctx->nb, ctx->K, ctx->J, elem_bytes(prec), bc, tile_bits, pd,
+    const int np = plan_hv_passes(ctx->n, pb, ctx->nb, ctx->K, ctx->J, elem_bytes(prec), 1, tile_bits, pd,
                                   FTK_MAX_PASSES, &pl.tile_bits, &pl.chunk_bits, 32, local_steps);
     if (np == 0) return false;
-    for (int p = 0; p < np; ++p)
-        if (!hv_layout_pass(pd[p], prec, bc)) return false;
+    if (hv_tiled(prec, pd[0])) {
+        for (int p = 0; p < np; ++p)
+            if (!hv_layout_pass(pd[p], prec)) return false;
+        pl.fix = prec == 0 && fix_plan(pd, np, pb, ctx->nb, ctx->K, ctx->J);
+    } else {
+        pl.gathers.resize(np);
+        for (int p = 0; p < np; ++p) gather_pass(pd[p], &pl.gathers[p]);
+    }
     pl.passes.assign(pd, pd + np);
-    pl.threads = hv_threads(pl.passes[0]);
-    pl.smem = hv_smem_bytes(prec, bc, pl.passes[0]);
     pl.grid = 8 * ctx->n_sm;   // cap of the persistent grid (4 MB of reduction partials)
-    return pl.smem <= (size_t(227) << 10);
+    return true;
 }
 
-bool plan_passes(ftk_ctx *ctx, int prec, int bc, int tile_bits, Plan &pl) {
-    if (plan_passes_with(ctx, prec, bc, tile_bits, kPlanLocalSteps, pl)) return true;
-    pl = Plan{};
-    return plan_passes_with(ctx, prec, bc, tile_bits, 0, pl);
+Plan whole_gather(const ftk_ctx *ctx) {
+    Plan pl;
+    pl.gathers.assign(1, ctx->gd);
+    pl.tile_bits = ctx->n;
+    return pl;
 }
 
 ftk_status get_plan(ftk_ctx *ctx, int prec, int B, Plan **out) {
     auto it = ctx->plans.find(prec * 64 + B);
     if (it != ctx->plans.end()) { *out = &it->second; return FTK_OK; }
-    if (ctx->tile_bits_req <= 0 && hv_use_gather(prec, ctx->n, B)) {
-        Plan pl;
-        pl.gather = true;
-        pl.tile_bits = ctx->n;
-        *out = &ctx->plans.emplace(prec * 64 + B, pl).first->second;
-        return FTK_OK;
-    }
-    // default: all columns in one launch (at most hv_max_b), the largest tile;
-    // the FP32 products of a relaxed double-float solve: one column per
-    // launch (the largest tile, fewest passes)
-    const int bc = (prec == FTK_FP32 && ctx->prec == FTK_DF) ? 1 : std::min(B, hv_max_b(prec));
-    const int tb_max = hv_max_tile_bits(prec, bc);
-    int tb = ctx->tile_bits_req > 0 ? std::min(ctx->tile_bits_req, tb_max) : tb_max;
-    tb = std::max(2, std::min(tb, ctx->n));
     Plan pl;
-    if (!plan_passes(ctx, prec, bc, tb, pl))
-        return fail(ctx, FTK_EINVAL, "H.v pass planning failed (tile too small for the bond list)");
-    auto res = ctx->plans.emplace(prec * 64 + B, pl);
-    *out = &res.first->second;
+    if (ctx->tile_bits_req <= 0 && hv_use_gather(prec, ctx->n, B)) {
+        pl = whole_gather(ctx);
+    } else {   // default: the largest tile
+        const int tb_max = hv_max_tile_bits(prec);
+        int tb = ctx->tile_bits_req > 0 ? std::min(ctx->tile_bits_req, tb_max) : tb_max;
+        tb = std::max(2, std::min(tb, ctx->n));
+        if (!plan_passes(ctx, prec, tb, pl))
+            return fail(ctx, FTK_EINVAL, "H.v pass planning failed (tile too small for the bond list)");
+    }
+    *out = &ctx->plans.emplace(prec * 64 + B, pl).first->second;
     return FTK_OK;
 }
 
@@ -223,19 +223,33 @@ int upd_grid(ftk_ctx *ctx, int B) {
 
 // H.V over all passes. The last pass uses epilogue epi, earlier ones write
 // or accumulate the partial product into out.
+cudaError_t run_plan(ftk_ctx *ctx, const Plan &pl, int prec, int B, int epi, const void *in, void *out, EpiArgs ea) {
+    cudaError_t e = cudaSuccess;
+    for (const GatherDesc &g : pl.gathers) {
+        e = launch_hv_gather(prec, B, g.last ? epi : EPI_PLAIN, in, out, g, ea, ctx->stream);
+        if (e != cudaSuccess) return e;
+        ++ctx->launches;
+    }
+    if (!pl.gathers.empty()) return e;
+    if (pl.fix && !ea.range) {   // (a solve's updates measure their residuals)
+        e = launch_fix_range(in, ctx->dim, B, ctx->dsmall->range, ea, ctx->n_sm, ctx->stream);
+        if (e != cudaSuccess) return e;
+        ++ctx->launches;
+        ea.range = ctx->dsmall->range;
+    }
+    for (const PassDesc &p : pl.passes) {
+        e = launch_hv_pass(prec, B, p.last ? epi : EPI_PLAIN, in, out, p, ea, pl.grid, ctx->stream);
+        if (e != cudaSuccess) return e;
+        ++ctx->launches;
+    }
+    return e;
+}
+
 ftk_status run_hv(ftk_ctx *ctx, int prec, int B, int epi, const void *in, void *out, EpiArgs ea) {
     Plan *pl = nullptr;
     ftk_status s = get_plan(ctx, prec, B, &pl);
     if (s != FTK_OK) return s;
-    if (pl->gather) {
-        LAUNCH(launch_hv_gather(prec, B, epi, in, out, ctx->gd, ea, ctx->stream));
-        return FTK_OK;
-    }
-    const int np = (int)pl->passes.size();
-    for (int p = 0; p < np; ++p) {
-        const int e = (p == np - 1) ? epi : EPI_PLAIN;
-        LAUNCH(launch_hv_pass(prec, B, e, in, out, pl->passes[p], ea, pl->grid, ctx->stream));
-    }
+    CK(run_plan(ctx, *pl, prec, B, epi, in, out, ea));
     return FTK_OK;
 }
 
@@ -604,8 +618,8 @@ ftk_status ftk_set_probe(ftk_ctx *ctx, int32_t slot, const double *v, int32_t is
 // One blocked COCG iteration on the context stream (no host sync):
 // H R_cur -> W (+mu), seed scalars, shift recurrences, R_prev <- update. In
 // the double-float mode the order is shifted by one step: R_prev <- update
-// of the previous step inside the first pass of H R_prev -> W (+mu), seed
-// scalars, shift recurrences (step 0 runs before the captured loop).
+// of the previous step, H R_prev -> W (+mu), seed scalars, shift recurrences
+// (step 0 runs before the captured loop).
 // Kind of the update kernel: 0 FP64 vectors, 1 FP32 vectors, 2 mixed (split
 // float hi + lo residuals; hi at the buffer start, lo ua.lo_stride float2
 // elements later).
@@ -650,8 +664,10 @@ static ftk_status cocg_iteration(ftk_ctx *ctx, int B, void *rcur, void *rprev, v
         return FTK_OK;
     };
     if (ctx->prec == FTK_DF) {
-        // double-float: the update r_{k-1} <- r_{k+1} of the previous step runs
-        // inside the first pass of H r_{k+1} (rcur = r_k, rprev = r_{k-1})
+        // double-float: the update r_{k-1} <- r_{k+1} of the previous step, then
+        // H r_{k+1} (rcur = r_k, rprev = r_{k-1}). The update inside the first
+        // pass of the product moved the same bytes in the same time (264 us of
+        // 522 at 24 sites against 260 alone), and kept that pass at 16 warps.
         if (ctx->relax > 0.0) {
             // relaxed phase (device flag lowp): the update alone, then the
             // FP32 H.V of the hi parts with mu from hi + lo; the
@@ -674,25 +690,13 @@ static ftk_status cocg_iteration(ftk_ctx *ctx, int B, void *rcur, void *rprev, v
             ea.lowp_run = 0;
         }
         ea.df_lo = ua.lo_stride;
-        Plan *pl = nullptr;
-        ftk_status ps = get_plan(ctx, ctx->mprec, B, &pl);
+        UpdArgs u = ua;
+        u.mode = 1;
+        u.lowp = ea.lowp;
+        u.lowp_run = 0;
+        LAUNCH(launch_cocg_update(upd_kind(ctx), B, rcur, w, rprev, u, upd_grid(ctx, B), ctx->stream));
+        const ftk_status ps = run_hv(ctx, ctx->mprec, B, EPI_COCG, rprev, w, ea);
         if (ps) return ps;
-        if (pl->gather) {
-            // the gather reads its partners' finished residuals: the update
-            // is a launch of its own
-            UpdArgs u = ua;
-            u.mode = 1;
-            u.lowp = ea.lowp;
-            u.lowp_run = 0;
-            LAUNCH(launch_cocg_update(upd_kind(ctx), B, rcur, w, rprev, u, upd_grid(ctx, B), ctx->stream));
-            if ((ps = run_hv(ctx, ctx->mprec, B, EPI_COCG, rprev, w, ea))) return ps;
-        } else {
-            ea.fu_seed = ua.seed;
-            ea.fu_rcur = static_cast<float2 *>(rcur);
-            ea.fu_lam = ua.lam_split;
-            ea.fu_result = ua.result;
-            if ((ps = run_hv(ctx, ctx->mprec, B, EPI_COCG, rprev, w, ea))) return ps;
-        }
         ftk_status s = join();
         if (s) return s;
         LAUNCH(launch_cocg_seed(sa, ctx->stream));
@@ -835,6 +839,10 @@ static ftk_status cocg_core(ftk_ctx *ctx, const CocgReq &rq, double *G_out, int3
     ea.result = d->hv_dots;
     ea.all_done = &d->all_done;
     ea.col_seed = d->seed;
+    if (pl->fix) {
+        ua.range = d->range;
+        ea.range = d->range;
+    }
     SeedArgs sa{};
     sa.n_rhs = B;
     sa.max_iter = rq.max_iter;
@@ -1505,7 +1513,7 @@ ftk_status ftk_plan_info(const ftk_ctx *cctx, int32_t *n_passes, int32_t *tile_b
     Plan *pl = nullptr;
     ftk_status s = get_plan(ctx, ctx->mprec, 1, &pl);
     if (s) return s;
-    if (n_passes) *n_passes = pl->gather ? 1 : (int)pl->passes.size();
+    if (n_passes) *n_passes = pl->n_passes();
     if (tile_bits) *tile_bits = pl->tile_bits;
     return FTK_OK;
 }
@@ -1540,15 +1548,12 @@ ftk_status ftk_autotune(ftk_ctx *ctx, int32_t n_rhs, int32_t which, int32_t *til
     if (prec == 2) ea.df_lo = (long long)n_rhs * (long long)ctx->dim;
     ftk_status st = FTK_OK;
     auto time_plan = [&](const Plan &pl) {
-        for (int rep = 0; rep < 4; ++rep) {
+        const int64_t l0 = ctx->launches;
+        for (int rep = 0; rep < 4 && st == FTK_OK; ++rep) {
             if (rep == 1 && cudaEventRecord(e0, ctx->stream) != cudaSuccess) st = FTK_ECUDA;
-            if (pl.gather && launch_hv_gather(prec, n_rhs, EPI_PLAIN, in, out, ctx->gd, ea, ctx->stream) != cudaSuccess)
-                st = FTK_ECUDA;
-            for (size_t p = 0; p < pl.passes.size() && st == FTK_OK; ++p)
-                if (launch_hv_pass(prec, n_rhs, EPI_PLAIN, in, out, pl.passes[p], ea, pl.grid, ctx->stream) !=
-                    cudaSuccess)
-                    st = FTK_ECUDA;
+            if (run_plan(ctx, pl, prec, n_rhs, EPI_PLAIN, in, out, ea) != cudaSuccess) st = FTK_ECUDA;
         }
+        ctx->launches = l0;
         float ms = 0;
         if (st == FTK_OK && (cudaEventRecord(e1, ctx->stream) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess ||
                              cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess))
@@ -1556,26 +1561,19 @@ ftk_status ftk_autotune(ftk_ctx *ctx, int32_t n_rhs, int32_t which, int32_t *til
         const double us = 1e3 * ms / 3;
         if (st == FTK_OK && us < best_us) { best_us = us; best = pl; }
     };
-    for (int bc = 1; bc <= std::min((int)n_rhs, hv_max_b(prec)) && st == FTK_OK; bc <<= 1) {
-        const int tb_max = std::min(hv_max_tile_bits(prec, bc), ctx->n);
-        for (int tb = std::max(5, tb_max - 2); tb <= tb_max && st == FTK_OK; ++tb) {
-            Plan pl;
-            if (plan_passes(ctx, prec, bc, tb, pl)) time_plan(pl);
-        }
-    }
-    if (st == FTK_OK && hv_use_gather(prec, ctx->n, n_rhs)) {
+    const int tb_max = std::min(hv_max_tile_bits(prec), ctx->n);
+    for (int tb = std::max(5, tb_max - 2); tb <= tb_max && st == FTK_OK; ++tb) {
         Plan pl;
-        pl.gather = true;
-        pl.tile_bits = ctx->n;
-        time_plan(pl);
+        if (plan_passes(ctx, prec, tb, pl)) time_plan(pl);
     }
+    if (st == FTK_OK && hv_use_gather(prec, ctx->n, n_rhs)) time_plan(whole_gather(ctx));
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (st != FTK_OK) return fail(ctx, st, "ftk_autotune: CUDA error while timing");
-    if (best.passes.empty() && !best.gather) return fail(ctx, FTK_EINVAL, "ftk_autotune: no admissible plan");
+    if (best.n_passes() == 0) return fail(ctx, FTK_EINVAL, "ftk_autotune: no admissible plan");
     ctx->plans[prec * 64 + n_rhs] = best;
     if (tile_bits_out) *tile_bits_out = best.tile_bits;
-    if (cols_out) *cols_out = best.gather ? n_rhs : best.passes[0].cols;
+    if (cols_out) *cols_out = best.passes.empty() ? n_rhs : 1;
     if (us_out) *us_out = best_us;
     return FTK_OK;
 }
@@ -1594,12 +1592,11 @@ ftk_status ftk_suggest_order(int32_t n_sites, const ftk_bond *bonds, int32_t n_b
         pb[q] = {b.i, b.j, b.gamma};
     }
     const int prec = precision == FTK_FP64 ? 0 : precision == FTK_DF ? 2 : 1;
-    const int tb_max = hv_max_tile_bits(prec, n_rhs);
+    const int tb_max = hv_max_tile_bits(prec);
     int tb = tile_bits > 0 ? std::min((int)tile_bits, tb_max) : tb_max;
     tb = std::max(2, std::min(tb, (int)n_sites));
     int perm[FTK_MAX_SITES];
-    const int np = plan_suggest_order(n_sites, pb, n_bonds, elem_bytes(prec), std::min((int)n_rhs, hv_max_b(prec)), tb,
-                                      perm);
+    const int np = plan_suggest_order(n_sites, pb, n_bonds, elem_bytes(prec), 1, tb, perm);
     if (np == 0) return fail(nullptr, FTK_EINVAL, "ftk_suggest_order: planning failed");
     for (int s = 0; s < n_sites; ++s) perm_out[s] = perm[s];
     if (n_passes_out) *n_passes_out = np;

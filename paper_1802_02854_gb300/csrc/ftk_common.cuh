@@ -10,6 +10,32 @@
 #define FTK_MAX_OMEGA 4096
 #define FTK_RED_THREADS 256   // threads of the last-block reductions
 
+// The couplings for the fixed-point FP64 passes (ftk_hv_fix.cu).
+struct FixCoef {
+    int32_t kh, kl, jh, jl;   // K/4 and J/4: (kh 2^30 + kl) 2^(ec - 60)
+    int32_t lsh;              // left shift of the 53-bit significands
+    int32_t sr;               // right shift of a pass's product
+    int32_t ex;               // exponent of the result's quantum minus the input's largest
+};
+// Exponents of a vector's components (one per column).
+struct FixRange {
+    int32_t e0;               // largest biased exponent
+    int32_t wide;             // 1: floating-point pass
+    int32_t emax;             // accumulators of the measuring launch (zero between launches)
+    uint32_t ticket;
+    unsigned long long sum, cnt;
+};
+
+// Matrix elements by bond type: a bond of type g adds, for parallel (par) /
+// antiparallel (anti) spins i, j, the amplitude par[g] / anti[g] to
+// |x ^ 2^i ^ 2^j>, and +dgv (parallel) / -dgv (antiparallel) on the diagonal,
+// dgv[0] = J/4 for x and y bonds, dgv[1] = (J + K)/4 for z bonds. _f, _lo: float
+// hi and lo parts.
+struct TypeCoef {
+    double par[3], anti[3], dgv[2];
+    float par_f[3], anti_f[3], par_lo[3], anti_lo[3], dgv_f[2], dgv_lo[2];
+};
+
 // One tiled pass of H.v: a CTA owns 2^tile_bits amplitudes whose index bits
 // tile_pos[] vary while the bits free_pos[] are fixed by the CTA index.
 // Bonds with both sites among tile_pos are applied from shared memory.
@@ -26,39 +52,26 @@ struct PassDesc {
     int32_t pad;
     int32_t tile_pos[FTK_MAX_TILE_BITS];
     int32_t free_pos[FTK_MAX_SITES];
-    int32_t bi[FTK_MAX_PASS_BONDS];   // tile-offset bit of site i
-    int32_t bj[FTK_MAX_PASS_BONDS];   // tile-offset bit of site j
-    // Bond (i, j) of type gamma adds, for parallel (p) / antiparallel (a)
-    // spins i, j, the off-diagonal amplitude par/anti to |x ^ 2^i ^ 2^j> and
-    // +dg (p) / -dg (a) on the diagonal.
-    double par[FTK_MAX_PASS_BONDS];
-    double anti[FTK_MAX_PASS_BONDS];
-    float par_f[FTK_MAX_PASS_BONDS];    // the same in float for the FP32 kernels
-    float anti_f[FTK_MAX_PASS_BONDS];
-    float par_lo[FTK_MAX_PASS_BONDS];   // par - par_f, anti - anti_f: low parts of the
-    float anti_lo[FTK_MAX_PASS_BONDS];  // double-float kernel's coefficients
-    // The diagonal of a pass is dgv[0] c0 + dgv[1] c1 with integer counts
-    // c = sum over the pass's bonds of class dgc (+1 parallel, -1 antiparallel):
-    // class 0 = x and y bonds (J/4), class 1 = z bonds ((J + K)/4).
-    int32_t dgc[FTK_MAX_PASS_BONDS];
-    double dgv[2];
-    float dgv_f[2];
-    float dgv_lo[2];
-    // Thread layout of the kernel (filled by hv_layout_pass): a CTA of
-    // 2^(tile_bits - le) threads, thread t owns the tile offsets t + 2^tb k
-    // for k < 2^le (tb = tile_bits - le), i.e. the top le offset bits are
-    // register bits. Bonds are ordered by group: the bonds of group g have
-    // the partner-thread mask grp_tmask[g] (the thread bits of their two
-    // sites) and occupy [grp_end[g-1], grp_end[g]); the last group has mask 0
-    // (partners held by the thread itself, and the diagonal). bcase encodes
-    // the register-bit part of the bond mask: 0 none, 1 + a one bit a,
-    // 9 + 8a + b two bits a < b.
-    int32_t le;
-    int32_t cols;      // right-hand sides per launch (column chunk width)
+    int8_t bi[FTK_MAX_PASS_BONDS];    // tile-offset bit of site i
+    int8_t bj[FTK_MAX_PASS_BONDS];    // tile-offset bit of site j
+    int8_t gam[FTK_MAX_PASS_BONDS];   // bond type
+    // Kernel form of the bonds (hv_layout_pass, see BondWalk), sorted by class:
+    // type, swap of an FP32 pair, register part of the mask.
+    uint32_t fdesc[FTK_MAX_PASS_BONDS];
+    int32_t f_end[24];
+    uint32_t classes;
+    // Double-float form (ftk_hv_df.cu): bonds ordered by group, those of group g
+    // with the partner-thread mask grp_tmask[g] in [grp_end[g-1], grp_end[g]), the
+    // last group with mask 0; bcase encodes the register part of a bond's mask: 0
+    // none, 1 + a one bit a, 9 + 8a + b two bits a < b.
     int32_t n_groups;
     int32_t grp_tmask[FTK_MAX_PASS_BONDS + 1];
     int32_t grp_end[FTK_MAX_PASS_BONDS + 1];
     int8_t bcase[FTK_MAX_PASS_BONDS];
+    float par_f[FTK_MAX_PASS_BONDS], anti_f[FTK_MAX_PASS_BONDS];
+    float par_lo[FTK_MAX_PASS_BONDS], anti_lo[FTK_MAX_PASS_BONDS];
+    TypeCoef tc;
+    FixCoef fx;
 };
 
 namespace ftk {

@@ -7,6 +7,13 @@
 
 namespace ftk {
 
+// Programmatic dependent launch: the next launch of the chain may start (its
+// blocks take the SMs that this one leaves, and prepare their offsets and
+// coefficients) / wait until the previous launch has completed and its writes
+// are visible. A launch without the attribute makes both no-ops.
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ---------------------------------------------------------------- complex
 template <typename R> struct C2;
 template <> struct C2<double> { typedef double2 t; };
@@ -116,22 +123,10 @@ __device__ __forceinline__ double warp_sums(const double (&v)[ND]) {
 template <int ND>
 __device__ void block_reduce(double (&v)[ND], double *red) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    constexpr int NG = ND <= 8 ? ND : 8;   // values folded at a time
-    static_assert(ND % NG == 0, "");
-    double s[ND / NG];
-#pragma unroll
-    for (int g = 0; g < ND / NG; ++g) {
-        double a[NG];
-#pragma unroll
-        for (int d = 0; d < NG; ++d) a[d] = v[g * NG + d];
-        s[g] = warp_sums<NG>(a);
-    }
-    const int d = warp_sums_index<NG>(lane);
+    const double s = warp_sums<ND>(v);
+    const int d = warp_sums_index<ND>(lane);
     __syncthreads();
-    if (d < NG && (lane & ((1 << (5 - WarpFold<NG>::levels)) - 1)) == 0) {
-#pragma unroll
-        for (int g = 0; g < ND / NG; ++g) red[warp * ND + g * NG + d] = s[g];
-    }
+    if (d < ND && (lane & ((1 << (5 - WarpFold<ND>::levels)) - 1)) == 0) red[warp * ND + d] = s;
     __syncthreads();
     if (threadIdx.x < ND) {
         double s = 0.0;
@@ -170,30 +165,60 @@ __device__ bool last_block_reduce(const double *partials, unsigned int *counter,
     return true;
 }
 
-// Bond coefficients in the kernel's arithmetic type (no per-element conversion).
-template <typename R> struct Coef;
-template <> struct Coef<double> {
-    __device__ static __forceinline__ double par(const PassDesc &p, int l) { return p.par[l]; }
-    __device__ static __forceinline__ double anti(const PassDesc &p, int l) { return p.anti[l]; }
-    __device__ static __forceinline__ double dgv(const PassDesc &p, int c) { return p.dgv[c]; }
+// ------------------------------------------------------ exponents
+// The exponents of a column's components, gathered by the launch that writes or
+// reads it: largest, sum and number of the nonzero ones. Integer atomics:
+// order-independent. add*: at most 2^20 amplitudes per thread.
+struct RangeAcc {
+    int em = 0;
+    unsigned sum = 0, cnt = 0;
+    __device__ __forceinline__ void add(int e) { em = max(em, e); sum += e; cnt += e != 0; }
+    __device__ __forceinline__ void add_fp64(const double2 &a) {
+        add((__double2hiint(a.x) >> 20) & 0x7ff);
+        add((__double2hiint(a.y) >> 20) & 0x7ff);
+    }
+    // by all threads of each of the nblk blocks of the column; true in the last
+    // block's first thread, with the column's totals in r
+    __device__ bool publish(FixRange *r, unsigned nblk) {
+        __shared__ int s_em;
+        __shared__ unsigned long long s_sum, s_cnt;
+        if (threadIdx.x == 0) { s_em = 0; s_sum = 0; s_cnt = 0; }
+        __syncthreads();
+        em = __reduce_max_sync(0xffffffffu, em);
+        unsigned long long sum64 = sum, cnt64 = cnt;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            sum64 += __shfl_xor_sync(0xffffffffu, sum64, o);
+            cnt64 += __shfl_xor_sync(0xffffffffu, cnt64, o);
+        }
+        if ((threadIdx.x & 31) == 0) {
+            atomicMax(&s_em, em);
+            atomicAdd(&s_sum, sum64);
+            atomicAdd(&s_cnt, cnt64);
+        }
+        __syncthreads();
+        if (threadIdx.x != 0) return false;
+        atomicMax(&r->emax, s_em);
+        atomicAdd(&r->sum, s_sum);
+        atomicAdd(&r->cnt, s_cnt);
+        __threadfence();
+        if (atomicAdd(&r->ticket, 1u) != nblk - 1) return false;
+        __threadfence();
+        return true;
+    }
+    // The verdicts: all zero: any exponent does; else the mean distance from the
+    // largest exponent within the limit, and no exponent near the ends of the
+    // range (inf and NaN have the largest).
+    __device__ void publish_fp64(FixRange *r, unsigned nblk) {
+        if (!publish(r, nblk)) return;
+        const int e = atomicExch(&r->emax, 0);
+        const unsigned long long s = atomicExch(&r->sum, 0ull), n = atomicExch(&r->cnt, 0ull);
+        r->e0 = n ? e : 1023;
+        // within 4.5 bits; 256 bits below for the quanta, 64 above for the sums
+        r->wide = n != 0 && (e < 256 || e > 1982 || 2ull * ((unsigned long long)e * n - s) > 9ull * n);
+        r->ticket = 0;
+    }
 };
-template <> struct Coef<float> {
-    __device__ static __forceinline__ float par(const PassDesc &p, int l) { return p.par_f[l]; }
-    __device__ static __forceinline__ float anti(const PassDesc &p, int l) { return p.anti_f[l]; }
-    __device__ static __forceinline__ float dgv(const PassDesc &p, int c) { return p.dgv_f[c]; }
-};
-
-// acc += c p for a complex amplitude and a real coefficient: on sm_100 and
-// later, float pairs take one packed FMA (fma.rn.f32x2) for both components
-__device__ __forceinline__ void cfma(double c, const double2 &p, double2 &acc) {
-    acc.x = fma(c, p.x, acc.x);
-    acc.y = fma(c, p.y, acc.y);
-}
-__device__ __forceinline__ void cfma(float c, const float2 &p, float2 &acc) {
-    acc = __ffma2_rn(make_float2(c, c), p, acc);
-}
-__device__ __forceinline__ void cadd(const double2 &p, double2 &acc) { acc.x += p.x; acc.y += p.y; }
-__device__ __forceinline__ void cadd(const float2 &p, float2 &acc) { acc = __fadd2_rn(acc, p); }
 
 // ------------------------------------------------------ H.V epilogues
 // What the last launch of a product does with an amplitude v and its finished
@@ -202,18 +227,20 @@ __device__ __forceinline__ void cadd(const float2 &p, float2 &acc) { acc = __fad
 template <typename R, int EPI>
 struct HvEpilogue {
     typedef typename C2<R>::t cx;
-    R scale, ell, inv_n, tcoef;
-    __device__ explicit HvEpilogue(const EpiArgs &ea)
-        : scale(EPI == EPI_TPQ ? (R)(*ea.scale) : (R)1), ell((R)ea.ell), inv_n((R)ea.inv_n),
-          tcoef(EPI == EPI_TAYLOR ? (R)ea.tcoef : (R)0) {}
+    // s l and -s / N (mTPQ: s the state's scale; Taylor: s the term's coefficient):
+    // combined once, two operations a component instead of three on the FP64
+    // pipe, which bounds the last pass
+    R lv, hv;
+    __device__ explicit HvEpilogue(const EpiArgs &ea) {
+        const double s = EPI == EPI_TPQ ? *ea.scale : EPI == EPI_TAYLOR ? ea.tcoef : 0.0;
+        lv = (R)(s * ea.ell);
+        hv = (R)(-s * ea.inv_n);
+    }
     template <typename D>
     __device__ __forceinline__ void apply(const EpiArgs &ea, size_t i, const cx &v, const cx &w, cx *out, D *dot) const {
-        if constexpr (EPI == EPI_PLAIN) {
-            *out = w;
-        } else if constexpr (EPI == EPI_TPQ) {
+        if constexpr (EPI == EPI_TPQ) {
             // psi' = s (l v - H v / N);  <v|Hv>, |psi'|^2
-            const R yr = scale * (ell * v.x - inv_n * w.x);
-            const R yi = scale * (ell * v.y - inv_n * w.y);
+            const R yr = fma(hv, w.x, lv * v.x), yi = fma(hv, w.y, lv * v.y);
             *out = mk<R>(yr, yi);
             dot[0].fma2(v.x, w.x);
             dot[0].fma2(v.y, w.y);
@@ -222,8 +249,7 @@ struct HvEpilogue {
         } else if constexpr (EPI == EPI_TAYLOR) {
             // cTPQ Taylor term: t' = c (l v - H v / N), acc += t';
             // <v|Hv> (the energy of v), |acc|^2
-            const R yr = tcoef * (ell * v.x - inv_n * w.x);
-            const R yi = tcoef * (ell * v.y - inv_n * w.y);
+            const R yr = fma(hv, w.x, lv * v.x), yi = fma(hv, w.y, lv * v.y);
             *out = mk<R>(yr, yi);
             cx *ap = reinterpret_cast<cx *>(ea.taylor_acc) + i;
             cx a = *ap;
@@ -234,9 +260,15 @@ struct HvEpilogue {
             dot[0].fma2(v.y, w.y);
             dot[1].fma2(a.x, a.x);
             dot[1].fma2(a.y, a.y);
-        } else if constexpr (EPI == EPI_COCG) {
-            // W = H R;  mu = R^T W (bilinear)
-            *out = w;
+        } else {
+            *out = w;   // W = H R
+            dots(ea, i, v, w, dot);
+        }
+    }
+    // the dots of an epilogue that stores the product as it is
+    template <typename D>
+    __device__ __forceinline__ void dots(const EpiArgs &ea, size_t i, const cx &v, const cx &w, D *dot) const {
+        if constexpr (EPI == EPI_COCG) {   // mu = R^T W (bilinear)
             dot[0].fma2(v.x, w.x);
             dot[0].fma2(-v.y, w.y);
             dot[1].fma2(v.x, w.y);
@@ -244,7 +276,6 @@ struct HvEpilogue {
         } else if constexpr (EPI == EPI_COCG_MIXED) {
             // mixed mode: R = hi + lo, mu = R^T W with exact FMA two-products
             // and two-sums (double-float, ~48 bits) on the FP32 pipe
-            *out = w;
             const float2 lo = reinterpret_cast<const float2 *>(ea.lo)[i];
             dot[0].fma_hl(v.x, lo.x, w.x);
             dot[0].fma_hl(-v.y, -lo.y, w.y);
@@ -343,28 +374,24 @@ __device__ __forceinline__ void dfl_mac(dfl &acc, dfl a, dfl b) {
 // Renormalised pair of an accumulator (two-sum: no ordering assumption).
 __device__ __forceinline__ dfl dfl_renorm(dfl a) { return dfl_two_sum(a.hi, a.lo); }
 
-// Multiply-accumulate of a bond's term in the double-float product.
-// The real and imaginary components take the same operations with the same
-// coefficient, so every step runs on float pairs (re, im) as one packed
-// f32x2 instruction (sm_100 and later). No step negates an operand: a - b is
-// formed as fma(b, -1, a) (the same rounding as the subtraction) and the
-// product's error term from the negated coefficient -c_hi, so each complex
-// term costs 12 packed instructions. h, l: the (re, im) hi and lo parts of
-// the accumulator.
+// Multiply-accumulate of a bond's term in the double-float product. The real and
+// imaginary components take the same operations with the same coefficient, so
+// every step runs on float pairs (re, im) as one packed f32x2 instruction (sm_100
+// and later); no step negates an operand (a - b is fma(b, -1, a), the same
+// rounding). h, l: the (re, im) hi and lo parts of the accumulator.
 __device__ __forceinline__ float2 m1x2() { return make_float2(-1.f, -1.f); }
 __device__ __forceinline__ float2 fsub2(float2 a, float2 b) { return __ffma2_rn(b, m1x2(), a); }   // a - b
-// acc += c p, c = ch + cl, p = ph + pl; nch = -ch, ncl = -cl:
-//   p_hh = ch ph;  en = -(ch ph - p_hh) - ch pl - cl ph  (exact first step)
-//   t = h + p_hh, Knuth two-sum error into l together with -en
-__device__ __forceinline__ void df_acc2(float2 &h, float2 &l, float2 ch, float2 nch, float2 ncl, float2 ph, float2 pl) {
+// acc += c p, c = ch + cl, p = ph + pl; nch = -ch:
+//   p_hh = ch ph;  en = -(ch ph - p_hh) - ch pl  (exact first step)
+//   t = h + p_hh, Knuth two-sum error into l together with -en and cl ph
+__device__ __forceinline__ void df_acc2(float2 &h, float2 &l, float2 ch, float2 nch, float2 cl, float2 ph, float2 pl) {
     const float2 p = __fmul2_rn(ch, ph);
     float2 en = __ffma2_rn(nch, ph, p);
     en = __ffma2_rn(nch, pl, en);
-    en = __ffma2_rn(ncl, ph, en);
     const float2 t = __fadd2_rn(h, p);
     const float2 bb = fsub2(t, h);
-    const float2 s = __fadd2_rn(fsub2(h, fsub2(t, bb)), fsub2(p, bb));
-    l = __fadd2_rn(l, fsub2(s, en));
+    const float2 q = __fadd2_rn(fsub2(h, fsub2(t, bb)), fsub2(p, bb));
+    l = __fadd2_rn(l, fsub2(__ffma2_rn(cl, ph, q), en));
     h = t;
 }
 __device__ __forceinline__ void df_add_to2(float2 &h, float2 &l, float2 ph, float2 pl) {

@@ -8,7 +8,9 @@
 // launches), while here 2^n threads spread over all of them. The price is one
 // 16-byte L2 read per bond and amplitude instead of a shared-memory one, so
 // the tiles win again once the reads of a launch cost more than the passes'
-// launches and empty SMs (hv_use_gather, with both sides measured).
+// launches and empty SMs (hv_use_gather, with both sides measured). Passes
+// whose requested tiles are too small for the tiled kernels run here too, one
+// launch per pass over the pass's bonds.
 #include "ftk_common.cuh"
 #include "ftk_device.cuh"
 #include "ftk_kernels.h"
@@ -31,10 +33,11 @@ template <> struct GatherVec<0> {
     typedef double coef;
     double2 s = {0.0, 0.0};
     __device__ static amp load(const void *p, size_t i, long long) { return static_cast<const double2 *>(p)[i]; }
-    __device__ static coef c(const GatherDesc &g, int q, bool anti) { return anti ? g.anti[q] : g.par[q]; }
+    __device__ static coef c(const GatherDesc &g, int q, bool anti) { return anti ? g.tc.anti[q] : g.tc.par[q]; }
     __device__ void add(coef c, const amp &a) { s.x = fma(c, a.x, s.x); s.y = fma(c, a.y, s.y); }
+    __device__ void partial(const amp &a) { s.x += a.x; s.y += a.y; }
     __device__ void diag(const GatherDesc &g, int c0, int c1, const amp &a) {
-        add((double)c0 * g.dgv[0] + (double)c1 * g.dgv[1], a);
+        add((double)c0 * g.tc.dgv[0] + (double)c1 * g.tc.dgv[1], a);
     }
 };
 template <> struct GatherVec<1> {
@@ -42,10 +45,11 @@ template <> struct GatherVec<1> {
     typedef float coef;
     float2 s = {0.f, 0.f};
     __device__ static amp load(const void *p, size_t i, long long) { return static_cast<const float2 *>(p)[i]; }
-    __device__ static coef c(const GatherDesc &g, int q, bool anti) { return anti ? g.anti_f[q] : g.par_f[q]; }
+    __device__ static coef c(const GatherDesc &g, int q, bool anti) { return anti ? g.tc.anti_f[q] : g.tc.par_f[q]; }
     __device__ void add(coef c, const amp &a) { s = __ffma2_rn(make_float2(c, c), a, s); }
+    __device__ void partial(const amp &a) { s = __fadd2_rn(s, a); }
     __device__ void diag(const GatherDesc &g, int c0, int c1, const amp &a) {
-        add((float)c0 * g.dgv_f[0] + (float)c1 * g.dgv_f[1], a);
+        add((float)c0 * g.tc.dgv_f[0] + (float)c1 * g.tc.dgv_f[1], a);
     }
 };
 template <> struct GatherVec<2> {
@@ -58,15 +62,16 @@ template <> struct GatherVec<2> {
         return make_float4(a.x, a.y, b.x, b.y);
     }
     __device__ static coef c(const GatherDesc &g, int q, bool anti) {
-        return anti ? make_float2(g.anti_f[q], g.anti_lo[q]) : make_float2(g.par_f[q], g.par_lo[q]);
+        return anti ? make_float2(g.tc.anti_f[q], g.tc.anti_lo[q]) : make_float2(g.tc.par_f[q], g.tc.par_lo[q]);
     }
     __device__ void add(coef c, const amp &a) {
-        df_acc2(h, l, make_float2(c.x, c.x), make_float2(-c.x, -c.x), make_float2(-c.y, -c.y), make_float2(a.x, a.y),
+        df_acc2(h, l, make_float2(c.x, c.x), make_float2(-c.x, -c.x), make_float2(c.y, c.y), make_float2(a.x, a.y),
                 make_float2(a.z, a.w));
     }
+    __device__ void partial(const amp &a) { df_add_to2(h, l, make_float2(a.x, a.y), make_float2(a.z, a.w)); }
     __device__ void diag(const GatherDesc &g, int c0, int c1, const amp &a) {
-        const dfl d = dfl_add(dfl_mul({(float)c0, 0.f}, {g.dgv_f[0], g.dgv_lo[0]}),
-                              dfl_mul({(float)c1, 0.f}, {g.dgv_f[1], g.dgv_lo[1]}));
+        const dfl d = dfl_add(dfl_mul({(float)c0, 0.f}, {g.tc.dgv_f[0], g.tc.dgv_lo[0]}),
+                              dfl_mul({(float)c1, 0.f}, {g.tc.dgv_f[1], g.tc.dgv_lo[1]}));
         add(make_float2(d.hi, d.lo), a);
     }
     // the renormalised pair
@@ -118,12 +123,13 @@ __global__ void __launch_bounds__(128) hv_gather_kernel(const void *__restrict__
         const int c1 = gd.off[3] - gd.off[2] - 2 * anti[2];
         const typename V::amp v = V::load(in, base + x, ea.df_lo);
         acc.diag(gd, c0, c1, v);
+        if (!gd.first) acc.partial(V::load(out, base + x, ea.df_lo));
         if constexpr (PREC == 2) {
             const float4 w = acc.value();
             float2 *o = static_cast<float2 *>(out) + base + x;
             o[0] = make_float2(w.x, w.y);
             o[ea.df_lo] = make_float2(w.z, w.w);
-            if constexpr (EPI == EPI_COCG) {   // mu = r^T w (bilinear) from hi + lo
+            if (EPI == EPI_COCG && gd.last) {   // mu = r^T w (bilinear) from hi + lo
                 dot[0].fma_pair(v.x, v.z, w.x, w.z);
                 dot[0].fma_pair(-v.y, -v.w, w.y, w.w);
                 dot[1].fma_pair(v.x, v.z, w.y, w.w);
@@ -132,10 +138,11 @@ __global__ void __launch_bounds__(128) hv_gather_kernel(const void *__restrict__
         } else {
             typedef typename C2<R>::t cx;
             cx *o = static_cast<cx *>(out) + base + x;
-            HvEpilogue<R, EPI>(ea).apply(ea, base + x, v, acc.s, o, dot);
+            if (!gd.last) *o = acc.s;
+            else HvEpilogue<R, EPI>(ea).apply(ea, base + x, v, acc.s, o, dot);
         }
     }
-    if constexpr (EPI != EPI_PLAIN) {
+    if (EPI != EPI_PLAIN && gd.last) {
         double d[ND];
 #pragma unroll
         for (int q = 0; q < ND; ++q) d[q] = dot[q].get();
@@ -152,44 +159,52 @@ bool gather_desc(int n, const PlanBond *bonds, int nb, double K, double J, Gathe
     if (n < 2 || n > FTK_MAX_SITES || nb < 1 || nb > 2 * FTK_MAX_PASS_BONDS) return false;
     GatherDesc d{};
     d.n_sites = n;
+    d.first = d.last = 1;
+    d.tc = type_coefficients(K, J);
     int w = 0;
     for (int g = 0; g < 3; ++g) {
         d.off[g] = w;
         for (int q = 0; q < nb; ++q)
             if (bonds[q].g == g) d.mask[w++] = (1u << bonds[q].i) | (1u << bonds[q].j);
-        bond_coefficients(g, K, J, &d.par[g], &d.anti[g]);
-        d.par_f[g] = (float)d.par[g];
-        d.anti_f[g] = (float)d.anti[g];
-        d.par_lo[g] = (float)(d.par[g] - (double)d.par_f[g]);
-        d.anti_lo[g] = (float)(d.anti[g] - (double)d.anti_f[g]);
     }
     d.off[3] = w;
     if (w != nb) return false;
-    d.dgv[0] = J / 4;
-    d.dgv[1] = (J + K) / 4;
-    for (int c = 0; c < 2; ++c) {
-        d.dgv_f[c] = (float)d.dgv[c];
-        d.dgv_lo[c] = (float)(d.dgv[c] - (double)d.dgv_f[c]);
-    }
     *gd = d;
     return true;
 }
 
-// Where the line lies, us per product of B vectors, gather against the fastest
-// tiled plan (captured launches, K = -1, J = 0.1):
-//   FP64  12 sites 3.9 / 34, 16: 8.7 / 50, 18: 29 / 55, 20: 117 / 178; four
-//         vectors 4.0 / 54, 27 / 78, 107 / 156, 461 / 563: at 18 sites the
-//         gather runs at the FP64 pipe's rate
-//   FP32  12: 3.3 / 11, 16: 4.5 / 18, 18: 11 / 20, 20: 38 / 34; four vectors
-//         3.3 / 15, 10 / 19, 36 / 27, 143 / 73: from 2^19 amplitudes on the L2
-//         reads cost more than the passes
+void gather_pass(const PassDesc &pd, GatherDesc *gd) {
+    GatherDesc d{};
+    d.n_sites = pd.n_sites;
+    d.first = pd.first;
+    d.last = pd.last;
+    d.tc = pd.tc;
+    int w = 0;
+    for (int g = 0; g < 3; ++g) {
+        d.off[g] = w;
+        for (int q = 0; q < pd.n_bonds; ++q)
+            if (pd.gam[q] == g) d.mask[w++] = (1u << pd.tile_pos[pd.bi[q]]) | (1u << pd.tile_pos[pd.bj[q]]);
+    }
+    d.off[3] = w;
+    *gd = d;
+}
+
+// Where the line lies, us per product of B vectors, gather against the tiled
+// passes (K = -1, J = 0.1):
+//   FP64  18 sites 29 / 37, 20 sites 117 / 66; four vectors: 16 sites 27 / -,
+//         18 sites 107 / 64, 20 sites 461 / 192
+//   FP32  12 sites 3.3 / 11, 18: 11 / 15, 20: 38 / 31; four vectors: 16 sites
+//         10 / -, 18 sites 36 / 23, 20 sites 143 / -
 //   DF    12: 3.7 / 17, 16: 5.8 / 25, 18: 15 / 28, 20: 53 / 65; four vectors
-//         3.7 / 67, 14 / 99, 49 / 110, 201 / 293
+//         3.7 / 67, 14 / 99, 49 / 110, 201 / 187
+// (-: not measured). FP64 and FP32 cross between 2^18 and 2^19 amplitudes in
+// all, where the gather's L2 reads (and, in FP64, its multiply-adds at the FP64
+// pipe's rate) cost more than the passes' launches and empty SMs; the
+// double-float passes are dearer and cross above 2^20.
 bool hv_use_gather(int prec, int n, int B) {
-    if (prec != 1) return n <= 20;
     int w = n;
     for (int b = 1; b < B; b <<= 1) ++w;
-    return w <= 18;
+    return w <= (prec == 2 ? 20 : 18);
 }
 
 // Threads per block: few for the smallest vectors, so that their blocks reach
@@ -207,10 +222,12 @@ static cudaError_t launch_prec(int epi, dim3 grid, int threads, const void *in, 
         if constexpr (PREC == 1) hv_gather_kernel<1, EPI_COCG_MIXED><<<grid, threads, 0, st>>>(in, out, gd, ea);
         else return cudaErrorInvalidValue;
         break;
+       
     case EPI_TPQ:
         if constexpr (PREC == 0) hv_gather_kernel<0, EPI_TPQ><<<grid, threads, 0, st>>>(in, out, gd, ea);
         else return cudaErrorInvalidValue;
         break;
+       
     case EPI_TAYLOR:
         if constexpr (PREC == 0) hv_gather_kernel<0, EPI_TAYLOR><<<grid, threads, 0, st>>>(in, out, gd, ea);
         else return cudaErrorInvalidValue;

@@ -23,36 +23,25 @@ struct EpiArgs {
     double2 *taylor_acc;
     double tcoef;
     long long df_lo;         // double-float mode: float2 offset of the lo arrays of in and out
-    // Double-float mode, first pass of H r_{k+1}: the COCG residual update
-    // fused in (fu_seed != NULL). Per launch (one column): the pass's input
-    // r_{k+1} is computed tile by tile from r_k (fu_rcur), r_{k-1} (in place
-    // of which r_{k+1} is written: fu_rnew, the pass's `in`), w_k = H r_k (the
-    // pass's `out`, read before it is overwritten) and lambda split
-    // (fu_lam); rho, g, |r|^2 of r_{k+1} go to fu_result[0..5). Every pass
-    // of a column whose fu_seed is done returns at once.
     // Relaxed double-float solve: the launch runs only while *lowp equals
     // lowp_run (lowp NULL: always)
     const int *lowp;
     int lowp_run;
     // COCG: the right-hand sides' seed scalars; a finished column's products are
-    // skipped (NULL: none). The gather kernel's tickets are counter[column].
+    // skipped (NULL: none). The tickets of column j are counter[j].
     const CocgSeed *col_seed;
-    const CocgSeed *fu_seed;
-    float2 *fu_rcur;
-    float2 *fu_rnew;
-    const float4 *fu_lam;
-    double *fu_result;
+    const FixRange *range;   // FP64 passes: the columns' exponents (NULL: floating-point passes)
 };
 
-// Bonds of the one-launch product (ftk_gather.cu), sorted by type: those of
-// type g are mask[off[g] .. off[g + 1]), with the off-diagonal amplitude par /
-// anti (parallel / antiparallel spins) of the type; dgv as in PassDesc.
+// Bonds of a gather launch (ftk_gather.cu), sorted by type: those of type g are
+// mask[off[g] .. off[g + 1]). first: start from zero, else add to the partial
+// product in out; last: apply the epilogue.
 struct GatherDesc {
     int32_t n_sites;
+    int32_t first, last;
     int32_t off[4];
     uint32_t mask[2 * FTK_MAX_PASS_BONDS];
-    double par[3], anti[3], dgv[2];
-    float par_f[3], anti_f[3], par_lo[3], anti_lo[3], dgv_f[2], dgv_lo[2];
+    TypeCoef tc;
 };
 
 struct UpdArgs {
@@ -74,6 +63,7 @@ struct UpdArgs {
                              // written by mode 0, read by mode 1
     const int *lowp;         // relaxed solve: run only while *lowp == lowp_run (NULL: always)
     int lowp_run;
+    FixRange *range;         // FP64: the exponents of the new residuals, for their product (NULL: not wanted)
 };
 
 struct SeedArgs {
@@ -210,6 +200,24 @@ struct SpecArgs {
     int *trunc;              // [n_T]
 };
 
+// Launch whose kernel waits for the launch before it (wait_previous in
+// ftk_device.cuh) instead of starting after it: a chain of such launches hides
+// their latencies and prologues.
+template <typename... P, typename... A>
+cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A &&...args) {
+    cudaLaunchAttribute chain{};
+    chain.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    chain.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &chain;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<A &&>(args)...);
+}
+
 cudaError_t init_kernel_attributes();
 void set_thread_error(const char *msg);   // message for ftk_last_error(NULL)
 // What the momentum-sector code reads from a context.
@@ -227,23 +235,32 @@ struct CtxHam {
 struct ftk_ctx;
 namespace ftk {
 bool ctx_hamiltonian(ftk_ctx *c, CtxHam *h);
-// H.V pass (ftk_hv.cu). A planned pass is laid out once for the kernel's
-// thread layout and a column chunk width cols <= hv_max_b(prec)
-// (hv_layout_pass); a launch of B right-hand sides then runs B / cols column
-// chunks. grid_cap bounds the persistent grid (the size of ea.partials).
+// H.V pass (ftk_hv.cu) of B right-hand sides. A planned pass is laid out once
+// for the kernels (hv_layout_pass; false for tiles too small, which run as
+// gather launches). grid_cap bounds the persistent grid (the size of
+// ea.partials).
 cudaError_t launch_hv_pass(int prec, int B, int epi, const void *in, void *out, const PassDesc &pd,
                            const EpiArgs &ea, int grid_cap, cudaStream_t st);
+bool hv_tiled(int prec, const PassDesc &pd);
 struct PlanBond;
 bool gather_desc(int n, const PlanBond *bonds, int nb, double K, double J, GatherDesc *gd);
+void gather_pass(const PassDesc &pd, GatherDesc *gd);   // the bonds of a planned pass
 bool hv_use_gather(int prec, int n, int B);
 cudaError_t launch_hv_gather(int prec, int B, int epi, const void *in, void *out, const GatherDesc &gd,
                              const EpiArgs &ea, cudaStream_t st);
-bool hv_layout_pass(PassDesc &pd, int prec, int B);
-int hv_max_b(int prec);
-int hv_le(int prec, int B, int tile_bits, int chunk_bits);
-int hv_max_tile_bits(int prec, int B);
-int hv_threads(const PassDesc &pd);
-size_t hv_smem_bytes(int prec, int B, const PassDesc &pd);
+// FP64 passes in fixed point (ftk_hv_fix.cu): coefficients of a laid-out plan
+// (false: the plan has no fixed-point form), the exponents of B vectors.
+bool fix_plan(PassDesc *pd, int np, const PlanBond *bonds, int nb, double K, double J);
+cudaError_t launch_fix_range(const void *in, uint64_t dim, int B, FixRange *range, const EpiArgs &ea, int n_sm,
+                             cudaStream_t st);
+typedef void (*FixKernel)(const double2 *, double2 *, long long, PassDesc, EpiArgs);
+FixKernel fix_kernel(int epi, bool full);   // full: tiles of the largest size
+// Double-float passes (ftk_hv_df.cu).
+typedef void (*TileKernel)(const float2 *, float2 *, long long, PassDesc, EpiArgs);
+bool df_layout_pass(PassDesc &pd);
+TileKernel df_kernel(int epi, bool full);
+bool hv_layout_pass(PassDesc &pd, int prec);
+int hv_max_tile_bits(int prec);
 // kind: 0 FP64 vectors, 1 FP32 vectors, 2 mixed (split float hi + lo
 // residuals, float w, double lambda)
 cudaError_t launch_cocg_update(int kind, int B, void *rcur, const void *w, void *rprev_new,

@@ -37,6 +37,7 @@ struct NoallocScratch {
     unsigned int counter;
     unsigned int pad[3];
     double result[4];
+    FixRange range;                        // exponents of the input
     double stats[3];                       // u_k, logQ_k, <H^2>_k of the step
     double partials[kNoallocMaxGrid * 2];  // [grid][2] per-CTA dots
 };
@@ -100,11 +101,12 @@ extern "C" ftk_status ftk_tpq_step_noalloc(int32_t n_sites, const ftk_bond *bond
     const bool gather = hv_use_gather(0, n_sites, 1) && gather_desc(n_sites, pb, n_bonds, K, J, &gd);
     PassDesc pd[FTK_MAX_PASSES];
     int tb = 0, cb = 0;
-    const int np = gather ? 0 : plan_hv_passes(n_sites, pb, n_bonds, K, J, 16, 1, hv_max_tile_bits(0, 1), pd, FTK_MAX_PASSES,
+    const int np = gather ? 0 : plan_hv_passes(n_sites, pb, n_bonds, K, J, 16, 1, hv_max_tile_bits(0), pd, FTK_MAX_PASSES,
                                   &tb, &cb);
     if (np == 0 && !gather) return noalloc_fail(FTK_EINVAL, "ftk_tpq_step_noalloc: pass planning failed");
     for (int p = 0; p < np; ++p)
-        if (!hv_layout_pass(pd[p], 0, 1)) return noalloc_fail(FTK_EINVAL, "ftk_tpq_step_noalloc: pass layout failed");
+        if (!hv_layout_pass(pd[p], 0)) return noalloc_fail(FTK_EINVAL, "ftk_tpq_step_noalloc: pass layout failed");
+    const bool fix = !gather && fix_plan(pd, np, pb, n_bonds, K, J);
     const long grid = kNoallocMaxGrid;   // the launcher trims it to the resident CTAs
 
     // state of this step: normalised input (scale 1), log Q and k start at 0;
@@ -131,6 +133,14 @@ extern "C" ftk_status ftk_tpq_step_noalloc(int32_t n_sites, const ftk_bond *bond
     if (gather) {
         e = launch_hv_gather(0, 1, EPI_TPQ, psi_dev, out_dev, gd, ea, st);
         if (e != cudaSuccess) return noalloc_fail(FTK_ECUDA, cudaGetErrorString(e));
+    }
+    if (fix) {
+        int n_sm = 0;
+        e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+        if (e == cudaSuccess) e = cudaMemsetAsync(&s->range, 0, sizeof(FixRange), st);
+        if (e == cudaSuccess) e = launch_fix_range(psi_dev, uint64_t(1) << n_sites, 1, &s->range, ea, n_sm, st);
+        if (e != cudaSuccess) return noalloc_fail(FTK_ECUDA, cudaGetErrorString(e));
+        ea.range = &s->range;
     }
     for (int p = 0; p < np; ++p) {
         e = launch_hv_pass(0, 1, p == np - 1 ? EPI_TPQ : EPI_PLAIN, psi_dev, out_dev, pd[p], ea, (int)grid, st);

@@ -24,6 +24,24 @@ inline void bond_coefficients(int g, double K, double J, double *par, double *an
     else { *par = 0; *anti = J / 2; }
 }
 
+inline TypeCoef type_coefficients(double K, double J) {
+    TypeCoef t{};
+    for (int g = 0; g < 3; ++g) {
+        bond_coefficients(g, K, J, &t.par[g], &t.anti[g]);
+        t.par_f[g] = (float)t.par[g];
+        t.anti_f[g] = (float)t.anti[g];
+        t.par_lo[g] = (float)(t.par[g] - (double)t.par_f[g]);
+        t.anti_lo[g] = (float)(t.anti[g] - (double)t.anti_f[g]);
+    }
+    t.dgv[0] = J / 4;
+    t.dgv[1] = (J + K) / 4;
+    for (int c = 0; c < 2; ++c) {
+        t.dgv_f[c] = (float)t.dgv[c];
+        t.dgv_lo[c] = (float)(t.dgv[c] - (double)t.dgv_f[c]);
+    }
+    return t;
+}
+
 // Cover of the bonds by tile site sets (greedy, with seeded restarts).
 // Every tile keeps the chunk_bits lowest sites (contiguous runs of >= 256 B
 // for coalesced loads); the other sites of a pass are added one at a time,
@@ -117,19 +135,33 @@ inline bool plan_anneal_cover(int n, const PlanBond *bonds, int nb, int b, int c
     }
     for (int p = 0; p < np; ++p)
         for (int k = 0; k < m; ++k) mem[p][draw([&](int s) { return !chunk[s] && !mem[p][s]; })] = 1;
-    auto covered = [&]() {
+    auto bond_covered = [&](int q) -> int {
+        const int i = bonds[q].i, j = bonds[q].j;
+        for (int p = 0; p < np; ++p)
+            if ((chunk[i] || mem[p][i]) && (chunk[j] || mem[p][j])) return 1;
+        return 0;
+    };
+    // bonds at each site: a move changes the cover of those at its two sites only
+    int first_at[FTK_MAX_SITES + 1], at_site[4 * FTK_MAX_PASS_BONDS];
+    for (int s = 0, w = 0; s <= n; ++s) {
+        first_at[s] = w;
+        for (int q = 0; s < n && q < nb; ++q)
+            if (bonds[q].i == s || bonds[q].j == s) at_site[w++] = q;
+    }
+    auto covered_at = [&](int a, int x) {   // bonds at a or x that are covered
         int cov = 0;
-        for (int q = 0; q < nb; ++q) {
-            const int i = bonds[q].i, j = bonds[q].j;
-            for (int p = 0; p < np; ++p)
-                if ((chunk[i] || mem[p][i]) && (chunk[j] || mem[p][j])) { ++cov; break; }
+        for (int w = first_at[a]; w < first_at[a + 1]; ++w) cov += bond_covered(at_site[w]);
+        for (int w = first_at[x]; w < first_at[x + 1]; ++w) {
+            const int q = at_site[w];
+            if (bonds[q].i != a && bonds[q].j != a) cov += bond_covered(q);
         }
         return cov;
     };
-    int cur = covered();
+    int cur = 0;
+    for (int q = 0; q < nb; ++q) cur += bond_covered(q);
     double T = 2.0;
     for (long st = 0; st < steps && cur < nb; ++st) {
-        int kind, p = 0, a = -1, x = -1;
+        int kind, p = 0, a = -1, x = -1, before = 0;
         char moved[FTK_MAX_PASSES];
         if (joint_chunk && c > 0 && rng.next() % 10 == 0) {
             // a chunk site and a non-chunk site trade places (in every pass
@@ -137,6 +169,7 @@ inline bool plan_anneal_cover(int n, const PlanBond *bonds, int nb, int b, int c
             kind = 0;
             a = draw([&](int s) { return chunk[s] != 0; });
             x = draw([&](int s) { return !chunk[s]; });
+            before = covered_at(a, x);
             chunk[a] = 0;
             chunk[x] = 1;
             for (int q = 0; q < np; ++q) {
@@ -149,10 +182,11 @@ inline bool plan_anneal_cover(int n, const PlanBond *bonds, int nb, int b, int c
             p = (int)(rng.next() % (uint32_t)np);
             a = draw([&](int s) { return mem[p][s] != 0; });
             x = draw([&](int s) { return !chunk[s] && !mem[p][s]; });
+            before = covered_at(a, x);
             mem[p][a] = 0;
             mem[p][x] = 1;
         }
-        const int nw = covered();
+        const int nw = cur - before + covered_at(a, x);
         const double u = (double)(rng.next() >> 8) * (1.0 / 16777216.0);
         if (nw >= cur || u < exp((nw - cur) / T)) {
             cur = nw;
@@ -254,28 +288,15 @@ inline int plan_hv_passes(int n, const PlanBond *bonds, int nb, double K, double
         int taken = 0;
         for (int q = 0; q < nb && taken < FTK_MAX_PASS_BONDS; ++q) {
             if (!remaining[q] || !in_t[bonds[q].i] || !in_t[bonds[q].j]) continue;
-            double par, anti;
-            bond_coefficients(bonds[q].g, K, J, &par, &anti);
-            p.bi[taken] = tpos[bonds[q].i];
-            p.bj[taken] = tpos[bonds[q].j];
-            p.par[taken] = par;
-            p.anti[taken] = anti;
-            p.par_f[taken] = (float)par;
-            p.anti_f[taken] = (float)anti;
-            p.par_lo[taken] = (float)(par - (double)p.par_f[taken]);
-            p.anti_lo[taken] = (float)(anti - (double)p.anti_f[taken]);
-            p.dgc[taken] = bonds[q].g == 2 ? 1 : 0;
+            p.bi[taken] = (int8_t)tpos[bonds[q].i];
+            p.bj[taken] = (int8_t)tpos[bonds[q].j];
+            p.gam[taken] = (int8_t)bonds[q].g;
             remaining[q] = 0;
             ++taken;
         }
         if (taken == 0) continue;
         p.n_bonds = taken;
-        p.dgv[0] = J / 4;
-        p.dgv[1] = (J + K) / 4;
-        p.dgv_f[0] = (float)p.dgv[0];
-        p.dgv_f[1] = (float)p.dgv[1];
-        p.dgv_lo[0] = (float)(p.dgv[0] - (double)p.dgv_f[0]);
-        p.dgv_lo[1] = (float)(p.dgv[1] - (double)p.dgv_f[1]);
+        p.tc = type_coefficients(K, J);
         ++np;
     }
     for (int q = 0; q < nb; ++q)
