@@ -66,10 +66,10 @@ SOLVE_BYTES = {"fp64": 16, "df": 16, "mixed": 8, "fp32": 8}   # bytes per amplit
 DTYPE = {"fp64": "f64", "df": "f32x2 (double-float) H.v and Krylov vectors, f64 scalars",
          "mixed": "f32 H.v, f32x2 Krylov vectors, f64 scalars", "fp32": "f32 H.v, f64 scalars"}
 # FP32-pipe operations of the double-float H.v per amplitude and term (a bond
-# or the diagonal): two real double-float multiply-accumulates of 12
-# operations each (FMA two-product with the cross terms: 4; two-sum and the
-# lo update: 8)
-DF_OPS_PER_TERM = 24
+# or the diagonal): two real double-float multiply-accumulates of 10
+# operations each (product and two-sum: 5, one of them an FMA that also takes
+# in the product's error; cross terms and the lo update: 5)
+DF_OPS_PER_TERM = 20
 FP32_LANES_PER_SM = 128
 FP64_PEAK_TFLOPS = 1.25
 # DRAM bytes (read + write) of one double-float H.v of one column: ncu

@@ -381,17 +381,24 @@ __device__ __forceinline__ dfl dfl_renorm(dfl a) { return dfl_two_sum(a.hi, a.lo
 // rounding). h, l: the (re, im) hi and lo parts of the accumulator.
 __device__ __forceinline__ float2 m1x2() { return make_float2(-1.f, -1.f); }
 __device__ __forceinline__ float2 fsub2(float2 a, float2 b) { return __ffma2_rn(b, m1x2(), a); }   // a - b
-// acc += c p, c = ch + cl, p = ph + pl; nch = -ch:
-//   p_hh = ch ph;  en = -(ch ph - p_hh) - ch pl  (exact first step)
-//   t = h + p_hh, Knuth two-sum error into l together with -en and cl ph
+// acc += c p, c = ch + cl, p = ph + pl; nch = -ch. Knuth's two-sum of h and q =
+// fl(ch ph),
+//   t = fl(h + q), bb = fl(t - h), error (h - (t - bb)) + (q - bb),
+// with q - bb and the product's own error ch ph - q in one FMA, ch ph - bb
+// (rounded at 2^-24 of an ulp). The cross terms join the first half, which is
+// zero unless |q| > |h|, so that they round at their own size. 10 instructions;
+// with the product's error formed by itself, 12. Error of a product against
+// double-double, 24 sites: 4.58e-15 (with 12: 4.59e-15).
+// t subtracts -q: a product that enters an addition is contracted with it, and
+// t = fma(ch, ph, h) is no substitute (the two-sum needs a float addend; the
+// error was 8e-9).
 __device__ __forceinline__ void df_acc2(float2 &h, float2 &l, float2 ch, float2 nch, float2 cl, float2 ph, float2 pl) {
-    const float2 p = __fmul2_rn(ch, ph);
-    float2 en = __ffma2_rn(nch, ph, p);
-    en = __ffma2_rn(nch, pl, en);
-    const float2 t = __fadd2_rn(h, p);
+    const float2 t = fsub2(h, __fmul2_rn(nch, ph));
     const float2 bb = fsub2(t, h);
-    const float2 q = __fadd2_rn(fsub2(h, fsub2(t, bb)), fsub2(p, bb));
-    l = __fadd2_rn(l, fsub2(__ffma2_rn(cl, ph, q), en));
+    float2 e = fsub2(h, fsub2(t, bb));
+    e = __ffma2_rn(ch, pl, e);
+    e = __ffma2_rn(cl, ph, e);
+    l = __fadd2_rn(l, fsub2(e, __ffma2_rn(nch, ph, bb)));
     h = t;
 }
 __device__ __forceinline__ void df_add_to2(float2 &h, float2 &l, float2 ph, float2 pl) {

@@ -15,8 +15,9 @@
 // register bits). The group with mask 0 holds the bonds between register sites,
 // and the diagonal.
 //
-// What bounds it: the FP32 pipe, 12 packed f32x2 instructions a term (24 sites,
-// one vector: 752 us; 775 without chained launches). The layout of ftk_hv_tile.cuh (1024 threads, a
+// What bounds it: the FP32 pipe, 10 packed f32x2 instructions a term (24 sites,
+// one vector: 684 us, 18 T operations/s of the pipe's 40; 752 us with 12, 775
+// without chained launches). The layout of ftk_hv_tile.cuh (1024 threads, a
 // partner read per bond) ran 812 us against 752: its gain in latency
 // does not outweigh the extra instructions here. Exact float pieces (the sums of
 // ftk_hv_fix.cu on three aligned floats, 4.3 packed instructions a term) ran 959
@@ -314,14 +315,20 @@ bool df_layout_pass(PassDesc &pd) {
         const int bi = newpos[pd.bi[l]], bj = newpos[pd.bj[l]];
         tmask[l] = ((1 << bi) | (1 << bj)) & ((1 << tb) - 1);
     }
-    // distinct nonzero masks in first-appearance order, then 0
+    // distinct nonzero masks in first-appearance order, those of z bonds alone
+    // before or after the others (the smaller coefficients first: the partial
+    // sums are smaller and round less), then 0
+    const TypeCoef &tc = pd.tc;
+    const bool z_small = tc.anti[2] * tc.anti[2] <= tc.par[0] * tc.par[0] + tc.anti[0] * tc.anti[0];
     int gm[FTK_MAX_PASS_BONDS + 1], ng = 0;
-    for (int l = 0; l < nb; ++l) {
-        if (tmask[l] == 0) continue;
-        bool seen = false;
-        for (int g = 0; g < ng; ++g) seen |= gm[g] == tmask[l];
-        if (!seen) gm[ng++] = tmask[l];
-    }
+    for (const bool z : {true, false})
+        for (int l = 0; l < nb; ++l) {
+            if (tmask[l] == 0) continue;
+            bool seen = false, only_z = true;
+            for (int g = 0; g < ng; ++g) seen |= gm[g] == tmask[l];
+            for (int m = 0; m < nb; ++m) only_z &= tmask[m] != tmask[l] || pd.gam[m] == 2;
+            if (!seen && only_z == (z == z_small)) gm[ng++] = tmask[l];
+        }
     gm[ng++] = 0;
     int w = 0;
     for (int g = 0; g < ng; ++g) {
