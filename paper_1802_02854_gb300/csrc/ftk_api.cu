@@ -199,6 +199,14 @@ ftk_status get_plan(ftk_ctx *ctx, int prec, int B, Plan **out) {
         tb = std::max(2, std::min(tb, ctx->n));
         if (!plan_passes(ctx, prec, tb, pl))
             return fail(ctx, FTK_EINVAL, "H.v pass planning failed (tile too small for the bond list)");
+        // Few tiles per SM: tiles of half the size, two CTAs to an SM, if a
+        // greedy plan finds as few passes for them (20 sites, two FP32 vectors:
+        // 44 -> 35 us). With many tiles one CTA's copies run behind its own
+        // sums, and half tiles mean more passes.
+        if (prec != 2 && ctx->tile_bits_req <= 0 && ctx->n > tb && (B << (ctx->n - tb)) < 4 * ctx->n_sm) {
+            Plan half;
+            if (plan_passes(ctx, prec, tb - 1, half, 0) && half.n_passes() <= pl.n_passes()) pl = half;
+        }
     }
     *out = &ctx->plans.emplace(prec * 64 + B, pl).first->second;
     return FTK_OK;
