@@ -61,6 +61,11 @@ inline int plan_cover(int n, const PlanBond *bonds, int nb, int b, int c, uint32
     int n_rem = nb;
     for (int q = 0; q < nb; ++q) remaining[q] = 1;
     PlanRng rng{seed * 2654435761u + 12345u};
+    // bonds of each site: at[first[s]] .. at[first[s + 1] - 1]
+    int first[FTK_MAX_SITES + 1] = {}, at[4 * FTK_MAX_PASS_BONDS], fill[FTK_MAX_SITES];
+    for (int q = 0; q < nb; ++q) { ++first[bonds[q].i + 1]; ++first[bonds[q].j + 1]; }
+    for (int s = 0; s < n; ++s) { first[s + 1] += first[s]; fill[s] = first[s]; }
+    for (int q = 0; q < nb; ++q) { at[fill[bonds[q].i]++] = q; at[fill[bonds[q].j]++] = q; }
     int np = 0;
     while (n_rem > 0) {
         if (np >= max_passes) return 0;
@@ -68,25 +73,29 @@ inline int plan_cover(int n, const PlanBond *bonds, int nb, int b, int c, uint32
         memset(in2, 0, sizeof in2);
         int nt = 0;
         int *T = sets[np];
+        // per site: its remaining bonds, and those whose other site is in the tile
+        int touch[FTK_MAX_SITES] = {}, done[FTK_MAX_SITES] = {};
+        for (int q = 0; q < nb; ++q)
+            if (remaining[q]) { ++touch[bonds[q].i]; ++touch[bonds[q].j]; }
+        auto take = [&](int s) {
+            T[nt++] = s;
+            in2[s] = 1;
+            for (int a = first[s]; a < first[s + 1]; ++a) {
+                const int q = at[a];
+                if (remaining[q]) ++done[bonds[q].i == s ? bonds[q].j : bonds[q].i];
+            }
+        };
         const int start = (np == 0 && low_first) ? b : c;
-        for (int s = 0; s < start; ++s) { T[nt++] = s; in2[s] = 1; }
+        for (int s = 0; s < start; ++s) take(s);
         while (nt < b) {
             int best = -1;
             long best_score = -1;
             for (int s = 0; s < n; ++s) {
                 if (in2[s]) continue;
-                long done = 0, touch = 0;
-                for (int q = 0; q < nb; ++q) {
-                    if (!remaining[q] || (bonds[q].i != s && bonds[q].j != s)) continue;
-                    ++touch;
-                    const int other = bonds[q].i == s ? bonds[q].j : bonds[q].i;
-                    if (in2[other]) ++done;
-                }
-                const long score = (done * 1000 + touch) * 1024 + (seed ? (long)(rng.next() & 1023) : 0);
+                const long score = (done[s] * 1000l + touch[s]) * 1024 + (seed ? (long)(rng.next() & 1023) : 0);
                 if (score > best_score) { best_score = score; best = s; }
             }
-            T[nt++] = best;
-            in2[best] = 1;
+            take(best);
         }
         int taken = 0;
         for (int q = 0; q < nb; ++q)
