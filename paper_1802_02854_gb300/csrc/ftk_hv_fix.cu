@@ -27,8 +27,8 @@
 // 1.2e-16.
 //
 // What bounds it now: the issue slots and the integer pipe (24 sites, three
-// passes: 207, 225 and 246 us, 61-68 % of the issue slots and 47-54 % of the ALU;
-// 709 us per product for 2417).
+// passes: 203, 221 and 243 us, 61-68 % of the issue slots and 48-55 % of the ALU;
+// 709 us per product for 2417; a vector of wide range 2337).
 //
 // Layout and items as in ftk_hv_tile.cuh (1024 threads of 4 amplitudes: 32 warps
 // hide the latencies that 16 warps of 8 or 8 of 16 did not). The y bonds come

@@ -28,7 +28,7 @@
 // of the issue slots, 16 warps a SM. Here
 // 32 warps hide the latencies and a bond costs a dozen instructions per thread
 // beside its reads and terms. FP32, 24 sites: 282 -> 217 us a product (three
-// passes, 67-90 us, bound by the shared-memory pipe at 69 %); 26 sites 988 -> 853.
+// passes, 72-87 us, the shared-memory pipe 63-67 % busy); 26 sites 988 -> 853.
 #pragma once
 #include "ftk_common.cuh"
 #include "ftk_device.cuh"
