@@ -299,7 +299,8 @@ ftk_status ftk_spectrum_ex(ftk_ctx *ctx, const double *G, int32_t n_shell, int32
  * whose stabiliser chi is 1. A sector vector holds dim complex amplitudes
  * (FP64 (re, im)) in ascending order of r.
  * The sector owns its device memory (allocated by ftk_sector_create): 4 B per
- * full-basis state for the state -> (orbit, element) table, the orbit list,
+ * full-basis state for the state -> (orbit, element) table, the
+ * representative of every basis vector (4 B each), the orbit list,
  * and n_slots sector vectors; 9 B per full-basis state of temporary memory
  * during creation. Work runs on the context's stream.
  * ------------------------------------------------------------------------- */
