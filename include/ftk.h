@@ -385,7 +385,9 @@ ftk_status ftk_sector_combine(int32_t n_sec, int32_t n_steps, const double *logn
  * FTK_FP32 and FTK_MIXED; vector j at offset j 2^N; for FTK_DF the FP32 hi
  * parts [n_rhs][2^N] followed by the lo parts [n_rhs][2^N], value hi + lo).
  * v and out are device pointers, must not overlap, and
- * need 16-byte alignment. The product of Sec. IV.A's cost unit ("a Lanczos
+ * need 16-byte alignment. FTK_FP64: every component is within
+ * (n_bonds + 4) 2^-53 of the sum of its terms' sizes, as a chain of FP64
+ * multiply-adds (underflow apart). The product of Sec. IV.A's cost unit ("a Lanczos
  * step"); exposed for tests and the bandwidth metric. Asynchronous. */
 ftk_status ftk_hv(ftk_ctx *ctx, const void *v_dev, void *out_dev, int32_t n_rhs);
 

@@ -64,7 +64,7 @@ struct Small {
     unsigned int counters[8];
     unsigned int upd_counters[FTK_MAX_RHS];  // tickets of the updates' reductions, per column
     unsigned int hv_counters[FTK_MAX_RHS];   // tickets of the products' reductions, per column
-    FixRange range[FTK_MAX_RHS];             // exponents of the FP64 products' inputs
+    FixRange range[2][FTK_MAX_RHS];          // what was measured of the FP64 products' inputs, in turn
     double hv_dots[FTK_MAX_RHS * FTK_HV_DOTS];
     double upd_dots[FTK_MAX_RHS * FTK_UPD_DOTS];
     double op_dots[4];
@@ -76,7 +76,8 @@ struct Small {
 
 struct Plan {
     int tile_bits = 0, chunk_bits = 0, grid = 0;
-    bool fix = false;                // FP64: the passes have a fixed-point form
+    bool fix = false;                // FP64: the passes have a fixed-point form,
+    RangePlan range{};               // and this is its measuring launch
     // one launch per element where not empty: the whole vector (no passes), or
     // the passes of tiles too small for the tiled kernels
     std::vector<GatherDesc> gathers;
@@ -98,6 +99,10 @@ struct ftk_ctx {
     double K = 0, J = 0, ell_min = 0;
     std::vector<Bond> bonds;
     GatherDesc gd{};
+    // The next product measures into range[range_slot], which the launch before
+    // cleared. A captured solve holds an even number of products, so that the turns
+    // go on after any number of its launches.
+    int range_slot = 0;
     std::vector<double> pos;
     cudaStream_t stream = nullptr;
     bool own_stream = false;
@@ -170,7 +175,7 @@ bool plan_passes(ftk_ctx *ctx, int prec, int tile_bits, Plan &pl, long local_ste
     if (hv_tiled(prec, pd[0])) {
         for (int p = 0; p < np; ++p)
             if (!hv_layout_pass(pd[p], prec)) return false;
-        pl.fix = prec == 0 && fix_plan(pd, np, pb, ctx->nb, ctx->K, ctx->J);
+        pl.fix = prec == 0 && fix_plan(pd, np, pb, ctx->nb, ctx->K, ctx->J, &pl.range);
     } else {
         pl.gathers.resize(np);
         for (int p = 0; p < np; ++p) gather_pass(pd[p], &pl.gathers[p]);
@@ -239,11 +244,14 @@ cudaError_t run_plan(ftk_ctx *ctx, const Plan &pl, int prec, int B, int epi, con
         ++ctx->launches;
     }
     if (!pl.gathers.empty()) return e;
-    if (pl.fix && !ea.range) {   // (a solve's updates measure their residuals)
-        e = launch_fix_range(in, ctx->dim, B, ctx->dsmall->range, ea, ctx->n_sm, ctx->stream);
+    if (pl.fix) {
+        const int slot = ctx->range_slot;
+        e = launch_fix_range(in, ctx->n, B, ctx->dsmall->range[slot], ctx->dsmall->range[1 - slot], pl.range, ea, ctx->n_sm,
+                             ctx->stream);
         if (e != cudaSuccess) return e;
+        ctx->range_slot = 1 - slot;
         ++ctx->launches;
-        ea.range = ctx->dsmall->range;
+        ea.range = ctx->dsmall->range[slot];
     }
     for (const PassDesc &p : pl.passes) {
         e = launch_hv_pass(prec, B, p.last ? epi : EPI_PLAIN, in, out, p, ea, pl.grid, ctx->stream);
@@ -847,10 +855,6 @@ static ftk_status cocg_core(ftk_ctx *ctx, const CocgReq &rq, double *G_out, int3
     ea.result = d->hv_dots;
     ea.all_done = &d->all_done;
     ea.col_seed = d->seed;
-    if (pl->fix) {
-        ua.range = d->range;
-        ea.range = d->range;
-    }
     SeedArgs sa{};
     sa.n_rhs = B;
     sa.max_iter = rq.max_iter;
@@ -922,6 +926,7 @@ static ftk_status cocg_core(ftk_ctx *ctx, const CocgReq &rq, double *G_out, int3
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     const int64_t l0 = ctx->launches;
+    const int slot0 = ctx->range_slot;
     int64_t per_graph = 0;
     cudaError_t ce = cudaSuccess;
     {
@@ -933,6 +938,7 @@ static ftk_status cocg_core(ftk_ctx *ctx, const CocgReq &rq, double *G_out, int3
         if (cs == FTK_OK && cudaStreamWaitEvent(ctx->stream, ctx->ev_join, 0) != cudaSuccess)
             cs = fail(ctx, FTK_ECUDA, "joining the shift branch of the solve graph");
         ce = cudaStreamEndCapture(ctx->stream, &graph);
+        if (cs != FTK_OK || ce != cudaSuccess) ctx->range_slot = slot0;   // no product of the capture will run
         if (cs != FTK_OK) { if (graph) cudaGraphDestroy(graph); return cs; }
         CK(ce);
         per_graph = ctx->launches - l0;
@@ -1546,7 +1552,9 @@ ftk_status ftk_autotune(ftk_ctx *ctx, int32_t n_rhs, int32_t which, int32_t *til
     // scratch: two Krylov regions (each max_rhs vectors of the vector precision)
     void *in = wsp(ctx, ctx->L.kry[0]);
     void *out = wsp(ctx, ctx->L.kry[1]);
-    CK(cudaMemsetAsync(in, 0, ctx->dim * es * n_rhs, ctx->stream));
+    // equal components, which every form of the product takes (FP64: 4.8e-4, so that
+    // the passes run in fixed point)
+    CK(cudaMemsetAsync(in, 0x3f, ctx->dim * es * n_rhs, ctx->stream));
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));

@@ -16,14 +16,25 @@ struct FixCoef {
     int32_t lsh;              // left shift of the 53-bit significands
     int32_t sr;               // right shift of a pass's product
     int32_t ex;               // exponent of the result's quantum minus the input's largest
+    float need;               // admitted: vectors whose smallest sum is at least need 2^(emax + 1)
 };
-// Exponents of a vector's components (one per column).
+// What the measuring launch finds in a vector (one per column).
 struct FixRange {
-    int32_t e0;               // largest biased exponent
-    int32_t wide;             // 1: floating-point pass
-    int32_t emax;             // accumulators of the measuring launch (zero between launches)
-    uint32_t ticket;
-    unsigned long long sum, cnt;
+    int32_t emax;             // largest biased exponent of its components
+    uint32_t low;             // complement of the smallest sum's bf16 bits (starts from 0)
+};
+// Tiles and bonds of the measuring launch (fix_range_kernel in ftk_hv_fix.cu).
+// Bonds by which of the offset bits 0 and 1 they flip (none, 0, 1, both): places
+// of their own in mask, more of the first kind.
+constexpr int kRangeBits = 14, kRangeBonds = 31;
+__host__ __device__ constexpr int range_slots(int kind) { return kind == 0 ? 16 : 5; }
+__host__ __device__ constexpr int range_slot(int kind) { return kind == 0 ? 0 : 11 + 5 * kind; }
+struct RangePlan {
+    int32_t bits, n_free;     // a tile: 2^bits amplitudes
+    int32_t n[4];             // bonds of each kind
+    int32_t pos[kRangeBits], free_pos[FTK_MAX_SITES];
+    uint32_t mask[kRangeBonds];   // the other offset bits they flip (byte offset of the item)
+    uint32_t par, anti;       // lower bounds of the coefficients' sizes, bf16 twice
 };
 
 // Matrix elements by bond type: a bond of type g adds, for parallel (par) /

@@ -165,61 +165,6 @@ __device__ bool last_block_reduce(const double *partials, unsigned int *counter,
     return true;
 }
 
-// ------------------------------------------------------ exponents
-// The exponents of a column's components, gathered by the launch that writes or
-// reads it: largest, sum and number of the nonzero ones. Integer atomics:
-// order-independent. add*: at most 2^20 amplitudes per thread.
-struct RangeAcc {
-    int em = 0;
-    unsigned sum = 0, cnt = 0;
-    __device__ __forceinline__ void add(int e) { em = max(em, e); sum += e; cnt += e != 0; }
-    __device__ __forceinline__ void add_fp64(const double2 &a) {
-        add((__double2hiint(a.x) >> 20) & 0x7ff);
-        add((__double2hiint(a.y) >> 20) & 0x7ff);
-    }
-    // by all threads of each of the nblk blocks of the column; true in the last
-    // block's first thread, with the column's totals in r
-    __device__ bool publish(FixRange *r, unsigned nblk) {
-        __shared__ int s_em;
-        __shared__ unsigned long long s_sum, s_cnt;
-        if (threadIdx.x == 0) { s_em = 0; s_sum = 0; s_cnt = 0; }
-        __syncthreads();
-        em = __reduce_max_sync(0xffffffffu, em);
-        unsigned long long sum64 = sum, cnt64 = cnt;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            sum64 += __shfl_xor_sync(0xffffffffu, sum64, o);
-            cnt64 += __shfl_xor_sync(0xffffffffu, cnt64, o);
-        }
-        if ((threadIdx.x & 31) == 0) {
-            atomicMax(&s_em, em);
-            atomicAdd(&s_sum, sum64);
-            atomicAdd(&s_cnt, cnt64);
-        }
-        __syncthreads();
-        if (threadIdx.x != 0) return false;
-        atomicMax(&r->emax, s_em);
-        atomicAdd(&r->sum, s_sum);
-        atomicAdd(&r->cnt, s_cnt);
-        __threadfence();
-        if (atomicAdd(&r->ticket, 1u) != nblk - 1) return false;
-        __threadfence();
-        return true;
-    }
-    // The verdicts: all zero: any exponent does; else the mean distance from the
-    // largest exponent within the limit, and no exponent near the ends of the
-    // range (inf and NaN have the largest).
-    __device__ void publish_fp64(FixRange *r, unsigned nblk) {
-        if (!publish(r, nblk)) return;
-        const int e = atomicExch(&r->emax, 0);
-        const unsigned long long s = atomicExch(&r->sum, 0ull), n = atomicExch(&r->cnt, 0ull);
-        r->e0 = n ? e : 1023;
-        // within 4.5 bits; 256 bits below for the quanta, 64 above for the sums
-        r->wide = n != 0 && (e < 256 || e > 1982 || 2ull * ((unsigned long long)e * n - s) > 9ull * n);
-        r->ticket = 0;
-    }
-};
-
 // ------------------------------------------------------ H.V epilogues
 // What the last launch of a product does with an amplitude v and its finished
 // product w = (H v): store, and the dots of the mTPQ step, the Taylor term or

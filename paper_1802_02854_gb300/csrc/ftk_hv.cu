@@ -115,7 +115,7 @@ static cudaError_t init_attributes_once() {
             if (df_kernel(epi, full) && e == cudaSuccess) e = opt_in(df_kernel(epi, full));
             if (fix_kernel(epi, full) && e == cudaSuccess) e = opt_in(fix_kernel(epi, full));
         }
-    return e;
+    return e == cudaSuccess ? fix_attributes() : e;
 }
 
 cudaError_t init_kernel_attributes() {

@@ -16,25 +16,38 @@
 // two fixed-point multiplications by K/4 and J/4; the partial product between
 // passes is the 64-bit integer result, converted to double in the last one.
 //
-// Accuracy: the quantum is 2^-58 of the vector's largest component, so a term's
-// rounding is below that of the DFMA chain for every component above 2^-5 of
-// the largest, and the sums add none. fix_range_kernel measures that before
-// each product: the exponents of all nonzero components must lie within 4.5
-// bits of the largest on average (3.4 for a Gaussian vector at 24 sites), with
-// no infinity, NaN or extreme exponent. Any other vector takes the
-// floating-point pass (hv_tile_body), inside the same launches. Relative error
-// against a double-double product, Gaussian vectors: 6e-17, with the DFMA chain
-// 1.2e-16.
+// Accuracy: the quantum q is 2^-(53 + lsh) of 2^(e0 + 1), the power of two above
+// the vector's largest component (lsh: 5 with up to 10 bonds in a pass, 4 up to
+// 21, 3 up to 42), the sums add no rounding, and a component far below the largest
+// has only the digits above q. An output is as good as that of a chain of
+// multiply-adds only if its own terms are large against q, and outputs differ: a
+// vector may hold blocks of H, or single neighbourhoods, of tiny components. So
+// fix_range_kernel measures before each product, for every output and for real and
+// imaginary parts apart, a lower bound of the sum of its terms' sizes, and a vector
+// is admitted where the fixed-point error bound stays at every output within that
+// of the chain, (bonds + 1) 2^-53 of the sum (fix_plan). Any other vector (zeros or
+// tiny blocks, very wide ranges, extreme exponents, infinities, NaN) takes the
+// floating-point pass (hv_tile_body), inside the same launches. (Admission by the
+// mean distance of the exponents from the largest let blocks of tiny components
+// come out as 0.)
+//
+// Measured, relative to the norm of the product, against double-double sums, random
+// vectors, typical states and residuals at 18 to 24 sites: 6.0e-17 to 1.2e-16; the
+// chain of multiply-adds 8.6e-17 to 1.4e-16. At the worst component of any of them 3.8
+// 2^-53 of its terms; the chain 3.4, admission by the mean exponent 7.9.
 //
 // What bounds it now: the issue slots and the integer pipe (24 sites, three
-// passes: 203, 221 and 243 us, 61-68 % of the issue slots and 48-55 % of the ALU;
-// 709 us per product for 2417; a vector of wide range 2337).
+// passes: 208, 226 and 246 us, 61-68 % of the issue slots and 48-55 % of the ALU;
+// with the measuring launch 751 us per product for 2412; a vector that is not
+// admitted 2365; 18 sites, four vectors: 70 for 166, not admitted 175).
 //
 // Layout and items as in ftk_hv_tile.cuh (1024 threads of 4 amplitudes: 32 warps
 // hide the latencies that 16 warps of 8 or 8 of 16 did not). The y bonds come
 // first, so that their A -= p plus a doubled D turns into A += +-p by one
 // addition per amplitude. Shared memory: the next tile's doubles (cp.async),
 // the integers of the current one, and the next partial products, 64 KB each.
+#include <cuda_bf16.h>
+
 #include "ftk_common.cuh"
 #include "ftk_device.cuh"
 #include "ftk_hv_tile.cuh"
@@ -43,42 +56,148 @@
 
 #include <algorithm>
 #include <math.h>
+#include <string.h>
+#include <type_traits>
 
 namespace ftk {
 
-// ---------------------------------------------------------------- exponents
-// Exponents of a vector's components (grid (blocks, columns)).
-__global__ void __launch_bounds__(256) fix_range_kernel(const double2 *__restrict__ in, uint64_t dim, FixRange *range,
-                                                        const int *all_done, const CocgSeed *col_seed) {
+// ---------------------------------------------------------------- measuring
+// Largest exponent of a vector's components and the smallest of its outputs'
+// sums of term sizes, over the x and y bonds inside tiles of 2^14 amplitudes (12
+// to 14 bonds on the honeycomb clusters; a term left out only lowers the bound).
+// Grid (split x persistent CTAs, columns): the outputs of a tile are shared by
+// split CTAs that all load it. A tile is held as bf16 sizes (rounded down, so that
+// the sums stay lower bounds; FixCoef::need holds the additions' rounding), four
+// neighbouring amplitudes in 16 bytes. Sizes below the float range count as 0,
+// which refuses.
+// What bounds it: at 24 sites the read (50 us of 74) and, after it, the shared reads
+// of 4 bytes a bond and amplitude (128 bytes a cycle and SM); below 20 sites one
+// tile's time, which split shortens.
+constexpr int kRangeThreads = 1024, kRangeCtas = 2, kRangeE = (1 << (kRangeBits - 2)) / kRangeThreads;   // items a thread
+// the bf16 bits of a double's size, from its upper word (right below 2^128)
+__device__ __forceinline__ int bf16_size(int hi) { return max((int)((unsigned)hi << 1 >> 14) - (896 << 7), 0); }
+__device__ __forceinline__ __nv_bfloat162 bf16x2(uint32_t u) { return *reinterpret_cast<__nv_bfloat162 *>(&u); }
+
+__global__ void __launch_bounds__(kRangeThreads, kRangeCtas)
+fix_range_kernel(const double2 *__restrict__ in, long long ld, const __grid_constant__ RangePlan rp, FixRange *range,
+                 FixRange *other, int split, const int *all_done, const CocgSeed *col_seed) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ uint32_t odd_k[kRangeE], ofs_k[4 * kRangeE], s_low;
+    __shared__ int s_em;
     launch_dependents();
+    const int t = threadIdx.x, T = blockDim.x, tb = 31 - __clz(T), n_k = 1 << (rp.bits - 2 - tb);
+    // offset of the thread's first amplitude in a tile, and the parities of its item
+    // bits with the bonds' masks; both for the bits above the thread's
+    uint32_t ofs = 0, odd = 0;
+    for (int q = 0; q < tb; ++q)
+        if ((t >> q) & 1) ofs |= 1u << rp.pos[q];
+    for (int q = 0; q < kRangeBonds; ++q) odd |= (uint32_t)(__popc(t * 16 & rp.mask[q]) & 1) << q;
+    if (t < 4 * n_k) {
+        uint32_t o = 0, p = 0;
+        for (int q = tb; q < rp.bits; ++q)
+            if ((t << tb >> q) & 1) o |= 1u << rp.pos[q];
+        ofs_k[t] = o;
+        if (t < n_k) {
+            for (int q = 0; q < kRangeBonds; ++q) p |= (uint32_t)(__popc((t << tb) * 16 & rp.mask[q]) & 1) << q;
+            odd_k[t] = p;
+        }
+    }
+    if (t == 0) { s_low = 0xffffffffu; s_em = 0; }
     wait_previous();
+    if (other && blockIdx.x == 0 && blockIdx.y == 0 && t < FTK_MAX_RHS) other[t] = FixRange{0, 0};
     if (all_done && *all_done) return;
     const int j = blockIdx.y;
     if (col_seed && col_seed[j].done != 0) return;
-    const double2 *v = in + (size_t)j * dim;
-    RangeAcc acc;
-    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    uint64_t x = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    for (; x + 3 * stride < dim; x += 4 * stride) {
-        const double2 a = v[x], b = v[x + stride], c = v[x + 2 * stride], d = v[x + 3 * stride];
-        acc.add_fp64(a); acc.add_fp64(b); acc.add_fp64(c); acc.add_fp64(d);
+    in += (size_t)j * ld + ofs;
+    const __nv_bfloat162 par = bf16x2(rp.par), anti = bf16x2(rp.anti);
+    __nv_bfloat162 low = bf16x2(0x7f807f80u);
+    int em = 0;
+    const int per = max(n_k / split, 1), k0 = (int)(blockIdx.x % split) * per;   // the CTA's items
+    for (uint32_t tau = blockIdx.x / split; tau < 1u << rp.n_free; tau += gridDim.x / split) {
+        uint32_t base = 0;
+        for (int q = 0; q < rp.n_free; ++q)
+            if ((tau >> q) & 1) base |= 1u << rp.free_pos[q];
+        __syncthreads();   // the previous tile is read
+        const double2 *v = in + base;
+#pragma unroll 8
+        for (int k = 0; k < 4 * n_k; ++k) {
+            const double2 a = v[ofs_k[k]];
+            const int x = bf16_size(__double2hiint(a.x)), y = bf16_size(__double2hiint(a.y));
+            *reinterpret_cast<uint32_t *>(smem_raw + 4 * (t + k * T)) = __byte_perm(x, y, 0x5410);
+            em = max(em, max(x, y));
+        }
+        __syncthreads();
+        for (int k = k0; k < k0 + per; k += 2) {   // two items at a time (twice the same if there is one)
+            const int k1 = min(k + 1, k0 + per - 1);
+            const uint32_t at[2] = {16u * (t + k * T), 16u * (t + k1 * T)};
+            const uint32_t w[2] = {odd ^ odd_k[k], odd ^ odd_k[k1]};
+            __nv_bfloat162 s[2][4];
+#pragma unroll
+            for (int x = 0; x < 8; ++x) s[x >> 2][x & 3] = bf16x2(0);
+            // the partner of word x of an item is word x ^ KIND of the partner item,
+            // and its parity the items' with that of x & KIND; unrolled, so that masks
+            // and parity bits are operands of one instruction each
+            const auto walk = [&](auto kind) {
+                constexpr int KIND = decltype(kind)::value;
+#pragma unroll
+                for (int u = 0; u < range_slots(KIND); ++u) {
+                    if (u >= rp.n[KIND]) break;
+                    constexpr int q0 = range_slot(KIND);
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) {
+                        const uint4 p4 = *reinterpret_cast<const uint4 *>(smem_raw + (at[i] ^ rp.mask[q0 + u]));
+                        const uint32_t p[4] = {p4.x, p4.y, p4.z, p4.w};
+                        const bool o = (w[i] & (1u << (q0 + u))) != 0;
+                        const __nv_bfloat162 c = o ? anti : par, f = o ? par : anti;
+#pragma unroll
+                        for (int x = 0; x < 4; ++x)
+                            s[i][x] = __hfma2(((x & KIND & 1) != 0) != ((x & KIND & 2) != 0) ? f : c,
+                                              bf16x2(p[x ^ KIND]), s[i][x]);
+                    }
+                }
+            };
+            walk(std::integral_constant<int, 0>());
+            walk(std::integral_constant<int, 1>());
+            walk(std::integral_constant<int, 2>());
+            walk(std::integral_constant<int, 3>());
+#pragma unroll
+            for (int x = 0; x < 8; ++x) low = __hmin2(low, s[x >> 2][x & 3]);
+        }
     }
-    for (; x < dim; x += stride) acc.add_fp64(v[x]);
-    acc.publish_fp64(range + j, gridDim.x);
+    // integer reductions: order-independent (positive floats order as integers)
+    const uint32_t lw = *reinterpret_cast<const uint32_t *>(&low);
+    em = __reduce_max_sync(0xffffffffu, em);
+    const uint32_t lmin = __reduce_min_sync(0xffffffffu, min(lw & 0xffffu, lw >> 16));
+    if ((t & 31) == 0) {
+        atomicMax(&s_em, em);
+        atomicMin(&s_low, lmin);
+    }
+    __syncthreads();
+    if (t == 0) {
+        atomicMax(&range[j].emax, (s_em >> 7) + 896);
+        atomicMax(&range[j].low, ~s_low);
+    }
+}
+// Whether a column takes fixed point: its largest component well inside the float
+// range (no infinity or NaN), and every output's sum as large as need asks.
+__device__ __forceinline__ bool fix_admits(const FixRange &r, float need) {
+    return r.emax >= 920 && r.emax <= 1120 &&
+           __uint_as_float(~r.low << 16) >= need * __uint_as_float((uint32_t)(r.emax + 1 - 896) << 23);
 }
 
 // ---------------------------------------------------------------- arithmetic
 // v as an integer: its 53-bit significand shifted to the common exponent e0
-// (|v| < 2^(e0 + 1 - 1023) maps below 2^(53 + lsh)), rounded toward zero.
+// (|v| < 2^(e0 + 1 - 1023) maps to at most 2^(53 + lsh)), rounded to nearest.
 __device__ __forceinline__ long long to_fixed(double v, int e0, int lsh) {
     const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
     const int sh = min(e0 - (int)((hi >> 20) & 0x7ffu), 63);   // zero: shifted out
-    const unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32 | lo) << lsh;
-    const long long s = (long long)(m >> sh);
+    const unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32 | lo) << (lsh + 1);
+    const long long s = (long long)((m >> sh) + 1) >> 1;
     return (int)hi < 0 ? -s : s;
 }
 // (K/4) A + (J/4) B in units of the result's quantum, from signed 32-bit digits
-// (the lowest digit product is below one quantum and dropped)
+// (the lowest digit products are dropped: with the roundings of the others less
+// than 1 + (kl + jl) 2^-31 quanta, and one more for a shift)
 __device__ __forceinline__ long long fix_combine(long long A, long long B, const FixCoef &f) {
     const int Al = (int)A, Bl = (int)B;
     const int Ah = (int)(A >> 32) - (Al >> 31), Bh = (int)(B >> 32) - (Bl >> 31);
@@ -133,7 +252,7 @@ __device__ __forceinline__ void bonds_fix(longlong2 (&A)[kTileE], longlong2 (&D)
 }
 
 // ---------------------------------------------------------------- the pass
-// Returns false, having done nothing, for a vector of wide range.
+// Returns false, having done nothing, for a vector that is not admitted.
 template <int EPI, int TB>
 __device__ __forceinline__ bool hv_fix_body(const double2 *__restrict__ in, double2 *out, const PassDesc &pd,
                                             const EpiArgs &ea0, long long ld) {
@@ -155,8 +274,8 @@ __device__ __forceinline__ bool hv_fix_body(const double2 *__restrict__ in, doub
     wait_previous();
     EpiArgs ea;
     if (!hv_column(ea0, ea, ld)) return true;
-    if (ea0.range[blockIdx.y].wide) return false;
-    const int e0 = ea0.range[blockIdx.y].e0;
+    if (!fix_admits(ea0.range[blockIdx.y], pd.fx.need)) return false;
+    const int e0 = ea0.range[blockIdx.y].emax;
     in += (size_t)blockIdx.y * ld;
     out += (size_t)blockIdx.y * ld;
     const HvEpilogue<double, EPI> epi(ea);
@@ -273,12 +392,62 @@ hv_fix_kernel(const double2 *__restrict__ in, double2 *out, long long ld, const 
 }
 
 // ===================================================================== host
-// Coefficients and scales for the passes of one plan. Sums: with |F| < 2^fb and
-// at most nb bonds in a pass, |A| <= nb 2^fb and |B| <= 2 nb 2^fb stay below
-// 2^62. K/4 and J/4 are 61-bit integers at a common exponent ec. The result's
-// quantum is 2^(ec + 2 + sr) of the input's; sr keeps the whole product (at
-// most sum_b (|off-diagonal| + |diagonal|) max |v|) below 2^62.
-bool fix_plan(PassDesc *pd, int np, const PlanBond *bonds, int nb, double K, double J) {
+// The measuring launch's tile: the lowest sites (contiguous runs of 128 bytes),
+// and greedily the sites with the most x and y bonds into it; its bonds, by which
+// of the sites 0 and 1 (the bits inside an item) they flip. Returns false if it
+// holds none.
+static bool range_plan(int n, const PlanBond *bonds, int nb, RangePlan *rp) {
+    RangePlan r{};
+    r.bits = std::min(n, kRangeBits);
+    r.n_free = n - r.bits;
+    int at[FTK_MAX_SITES];   // offset bit of a site, -1: not in the tile
+    std::fill(at, at + FTK_MAX_SITES, -1);
+    for (int w = 0; w < r.bits; ++w) {
+        int best = w, most = -1;
+        if (w >= 3) {
+            int score[FTK_MAX_SITES] = {};
+            for (int q = 0; q < nb; ++q) {
+                if (bonds[q].g == 2) continue;
+                score[bonds[q].i] += at[bonds[q].j] >= 0 ? 17 : 1;
+                score[bonds[q].j] += at[bonds[q].i] >= 0 ? 17 : 1;
+            }
+            for (int s = 0; s < n; ++s)
+                if (at[s] < 0 && score[s] > most) { most = score[s]; best = s; }
+        }
+        at[best] = w;
+    }
+    int f = 0;
+    for (int s = 0, w = 0; s < n; ++s) {   // ascending offset bits
+        if (at[s] < 0) { r.free_pos[f++] = s; continue; }
+        r.pos[w] = s;
+        at[s] = w++;
+    }
+    int total = 0;
+    for (int q = 0; q < nb; ++q) {
+        const int i = at[bonds[q].i], j = at[bonds[q].j];
+        if (bonds[q].g == 2 || i < 0 || j < 0) continue;
+        const uint32_t m = (1u << i) | (1u << j);
+        const int kind = m & 3;
+        if (r.n[kind] == range_slots(kind)) continue;
+        r.mask[range_slot(kind) + r.n[kind]++] = (m >> 2) * 16;
+        ++total;
+    }
+    *rp = r;
+    return total > 0;
+}
+
+// Coefficients and scales for the passes of one plan, and its measuring launch.
+// Sums: a pass of nb bonds adds at most nb amplitudes to A and 3 nb to B (the
+// antiparallel ones twice, and the diagonal), which has to stay below 2^63 with
+// room for the signed digits. K/4 and J/4 are 61-bit integers at a common exponent
+// ec. The result's quantum is 2^(ec + 2 + sr) of the input's; sr keeps the whole
+// product (at most sum_b (|off-diagonal| + |diagonal|) max |v|) below 2^62.
+// Admission, with q the input's quantum: an output's error is at most q / 2 for each
+// unit of its coefficients (at most bound in all), and per pass the roundings of
+// fix_combine. need is where that equals (nb + 1) 2^-53 of the sum of its terms'
+// sizes. The sum counts x and y bonds, so both of their coefficients must differ
+// from zero, else some state has no such term and no vector is admitted.
+bool fix_plan(PassDesc *pd, int np, const PlanBond *bonds, int nb, double K, double J, RangePlan *rp) {
     int most = 1;
     for (int p = 0; p < np; ++p) {
         pd[p].fx = FixCoef{};
@@ -287,40 +456,57 @@ bool fix_plan(PassDesc *pd, int np, const PlanBond *bonds, int nb, double K, dou
     }
     const double cmax = std::max(fabs(K), fabs(J)) / 4;
     if (!(cmax > 0x1p-40) || !(cmax < 0x1p40)) return false;   // exponents stay inside the range
+    double par, anti;
+    bond_coefficients(0, K, J, &par, &anti);
+    if (par == 0 || anti == 0 || !range_plan(pd[0].n_sites, bonds, nb, rp)) return false;
     int ec = 0;
     if (frexp(cmax, &ec) == 0.5) --ec;   // cmax <= 2^ec
     double bound = 0;
     for (int q = 0; q < nb; ++q) {
-        double par, anti;
-        bond_coefficients(bonds[q].g, K, J, &par, &anti);
-        bound += std::max(fabs(par), fabs(anti)) + fabs(bonds[q].g == 2 ? (J + K) / 4 : J / 4);
+        double p, a;
+        bond_coefficients(bonds[q].g, K, J, &p, &a);
+        bound += std::max(fabs(p), fabs(a)) + fabs(bonds[q].g == 2 ? (J + K) / 4 : J / 4);
     }
-    int lg = 0;
-    while ((1 << lg) < most) ++lg;
-    const int fb = 62 - lg;   // 2 most 2^fb <= 2^63 / ... : |B| < 2^63, its signed upper digit below 2^31
+    FixCoef f{};
+    while (3.0 * most * ldexp(1.0, 54 + f.lsh) <= 0x1p63 - 0x1p33) ++f.lsh;
     int eb = 0;
     frexp(bound, &eb);        // bound < 2^eb
-    FixCoef f{};
-    f.lsh = fb - 1 - 53;      // one bit of room for the signed digits
-    f.sr = std::max(0, eb + (fb - 1) - (ec + 2) - 62);
+    f.sr = std::max(0, eb + (53 + f.lsh) - (ec + 2) - 62);
     const long long ki = llrint(ldexp(K / 4, 60 - ec)), ji = llrint(ldexp(J / 4, 60 - ec));
     f.kh = (int)(ki >> 30);
     f.kl = (int)(ki & ((1 << 30) - 1));
     f.jh = (int)(ji >> 30);
     f.jl = (int)(ji & ((1 << 30) - 1));
-    f.ex = 1 - 1023 - (fb - 1) + ec + 2 + f.sr;
-    if (f.lsh < 0) return false;
+    f.ex = 1 - 1023 - (53 + f.lsh) + ec + 2 + f.sr;
+    // the coefficients' bf16 sizes, rounded down
+    const float cp = (float)fabs(par), ca = (float)fabs(anti);
+    auto below = [](float x) -> uint32_t {   // also where x itself was rounded up
+        uint32_t u;
+        memcpy(&u, &x, 4);
+        u = (u >> 16) > 0 ? (u >> 16) - 1 : 0;
+        return u << 16 | u;
+    };
+    rp->par = below(cp);
+    rp->anti = below(ca);
+    const double combine = 1 + ((double)f.kl + f.jl) * 0x1p-31 + (f.sr > 0);
+    const double need = (bound / 2 + np * combine * ldexp(1.0, ec + 2 + f.sr)) / (ldexp(1.0, f.lsh) * (nb + 1));
+    f.need = (float)(need * pow(1 + 0x1p-8, rp->n[0] + rp->n[1] + rp->n[2] + rp->n[3] + 2));   // bf16 additions, the float product
     for (int p = 0; p < np; ++p) pd[p].fx = f;
     return true;
 }
 
-cudaError_t launch_fix_range(const void *in, uint64_t dim, int B, FixRange *range, const EpiArgs &ea, int n_sm,
-                             cudaStream_t st) {
-    const uint64_t want = (dim + 1023) / 1024;
-    const uint64_t cap = std::max<uint64_t>(1, (uint64_t)8 * n_sm / B);
-    const dim3 grid((unsigned)std::min(want, cap), B);
-    return launch_chained(fix_range_kernel, grid, 256, 0, st, static_cast<const double2 *>(in), dim, range, ea.all_done,
-                          ea.col_seed);
+cudaError_t fix_attributes() {
+    return cudaFuncSetAttribute(fix_range_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 << kRangeBits);
+}
+cudaError_t launch_fix_range(const void *in, int n, int B, FixRange *range, FixRange *other, const RangePlan &rp,
+                             const EpiArgs &ea, int n_sm, cudaStream_t st) {
+    const int items = 1 << (rp.bits - 2), threads = std::min(kRangeThreads, items);
+    const int tiles = 1 << rp.n_free, resident = kRangeCtas * n_sm;
+    int split = 1;
+    while (split < items / threads && 2 * split * tiles * B <= n_sm) split *= 2;   // while SMs are idle
+    const int grid = std::min(tiles, std::max(1, resident / (split * B))) * split;
+    return launch_chained(fix_range_kernel, dim3(grid, B), threads, (size_t)items * 16, st,
+                          static_cast<const double2 *>(in), 1LL << n, rp, range, other, split, ea.all_done, ea.col_seed);
 }
 
 template <int TB>

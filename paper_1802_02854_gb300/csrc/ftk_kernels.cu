@@ -73,7 +73,6 @@ __global__ void __launch_bounds__(256) cocg_update_kernel(V vec, UpdArgs ua) {
     // range guard of the seed kernel: r_{k+1} and r_k (the next r_{k-1}) scaled by f
     const R f = ua.mode == 1 ? (R)ua.seed[j].rescale : (R)1;
     Acc<R> d_rr, d_ri, d_gr, d_gi, d_n;
-    RangeAcc range;
     if (!skip) {
         for (uint64_t x = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; x < n;
              x += (uint64_t)gridDim.x * blockDim.x) {
@@ -107,7 +106,6 @@ __global__ void __launch_bounds__(256) cocg_update_kernel(V vec, UpdArgs ua) {
                 }
             }
             vec.store(off + x, r);
-            if constexpr (sizeof(R) == 8) range.add_fp64(r);
             d_rr.fma2(r.x, r.x); d_rr.fma2(-r.y, r.y);
             d_ri.fma2(2 * r.x, r.y);
             d_gr.fma2(l.x, r.x); d_gr.fma2(l.y, r.y);
@@ -115,8 +113,6 @@ __global__ void __launch_bounds__(256) cocg_update_kernel(V vec, UpdArgs ua) {
             d_n.fma2(r.x, r.x); d_n.fma2(r.y, r.y);
         }
     }
-    if constexpr (sizeof(R) == 8)
-        if (ua.range) range.publish_fp64(ua.range + j, gridDim.x);
     double v[5] = {d_rr.get(), d_ri.get(), d_gr.get(), d_gi.get(), d_n.get()};
     block_reduce<5>(v, red);
     // the column's last block: fixed-order sum of its partials

@@ -30,7 +30,7 @@ struct EpiArgs {
     // COCG: the right-hand sides' seed scalars; a finished column's products are
     // skipped (NULL: none). The tickets of column j are counter[j].
     const CocgSeed *col_seed;
-    const FixRange *range;   // FP64 passes: the columns' exponents (NULL: floating-point passes)
+    const FixRange *range;   // FP64 passes: what was measured of the columns (NULL: floating-point passes)
 };
 
 // Bonds of a gather launch (ftk_gather.cu), sorted by type: those of type g are
@@ -63,7 +63,6 @@ struct UpdArgs {
                              // written by mode 0, read by mode 1
     const int *lowp;         // relaxed solve: run only while *lowp == lowp_run (NULL: always)
     int lowp_run;
-    FixRange *range;         // FP64: the exponents of the new residuals, for their product (NULL: not wanted)
 };
 
 struct SeedArgs {
@@ -249,10 +248,13 @@ bool hv_use_gather(int prec, int n, int B);
 cudaError_t launch_hv_gather(int prec, int B, int epi, const void *in, void *out, const GatherDesc &gd,
                              const EpiArgs &ea, cudaStream_t st);
 // FP64 passes in fixed point (ftk_hv_fix.cu): coefficients of a laid-out plan
-// (false: the plan has no fixed-point form), the exponents of B vectors.
-bool fix_plan(PassDesc *pd, int np, const PlanBond *bonds, int nb, double K, double J);
-cudaError_t launch_fix_range(const void *in, uint64_t dim, int B, FixRange *range, const EpiArgs &ea, int n_sm,
-                             cudaStream_t st);
+// and its measuring launch (false: the plan has no fixed-point form), the launch
+// for B vectors: range has to be zero, other (may be NULL) is cleared for the next
+// launch, once the products that read it are through.
+bool fix_plan(PassDesc *pd, int np, const PlanBond *bonds, int nb, double K, double J, RangePlan *rp);
+cudaError_t fix_attributes();
+cudaError_t launch_fix_range(const void *in, int n, int B, FixRange *range, FixRange *other, const RangePlan &rp,
+                             const EpiArgs &ea, int n_sm, cudaStream_t st);
 typedef void (*FixKernel)(const double2 *, double2 *, long long, PassDesc, EpiArgs);
 FixKernel fix_kernel(int epi, bool full);   // full: tiles of the largest size
 // Double-float passes (ftk_hv_df.cu).

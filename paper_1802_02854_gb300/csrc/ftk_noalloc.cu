@@ -37,7 +37,7 @@ struct NoallocScratch {
     unsigned int counter;
     unsigned int pad[3];
     double result[4];
-    FixRange range;                        // exponents of the input
+    FixRange range;                        // what was measured of the input
     double stats[3];                       // u_k, logQ_k, <H^2>_k of the step
     double partials[kNoallocMaxGrid * 2];  // [grid][2] per-CTA dots
 };
@@ -106,7 +106,8 @@ extern "C" ftk_status ftk_tpq_step_noalloc(int32_t n_sites, const ftk_bond *bond
     if (np == 0 && !gather) return noalloc_fail(FTK_EINVAL, "ftk_tpq_step_noalloc: pass planning failed");
     for (int p = 0; p < np; ++p)
         if (!hv_layout_pass(pd[p], 0)) return noalloc_fail(FTK_EINVAL, "ftk_tpq_step_noalloc: pass layout failed");
-    const bool fix = !gather && fix_plan(pd, np, pb, n_bonds, K, J);
+    RangePlan rp;
+    const bool fix = !gather && fix_plan(pd, np, pb, n_bonds, K, J, &rp);
     const long grid = kNoallocMaxGrid;   // the launcher trims it to the resident CTAs
 
     // state of this step: normalised input (scale 1), log Q and k start at 0;
@@ -138,7 +139,7 @@ extern "C" ftk_status ftk_tpq_step_noalloc(int32_t n_sites, const ftk_bond *bond
         int n_sm = 0;
         e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
         if (e == cudaSuccess) e = cudaMemsetAsync(&s->range, 0, sizeof(FixRange), st);
-        if (e == cudaSuccess) e = launch_fix_range(psi_dev, uint64_t(1) << n_sites, 1, &s->range, ea, n_sm, st);
+        if (e == cudaSuccess) e = launch_fix_range(psi_dev, n_sites, 1, &s->range, nullptr, rp, ea, n_sm, st);
         if (e != cudaSuccess) return noalloc_fail(FTK_ECUDA, cudaGetErrorString(e));
         ea.range = &s->range;
     }
