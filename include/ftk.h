@@ -309,7 +309,9 @@ typedef struct ftk_sector ftk_sector;
 /* perms: host [n_g][n_sites] (site l -> perms[g][l]), 1 <= n_g <= 32; chi: host
  * [n_g][2] (re, im). n_slots: sector vectors kept (1..64). *dim_out
  * receives the sector dimension. FTK_EINVAL if the permutations do not form
- * a group preserving the bonds, or chi is not a character of it. */
+ * a group preserving the bonds, chi is not a character of it, or the sector has
+ * 2^(32 - b) basis vectors or more, 2^b >= n_g (at 30 sites: groups of more than
+ * eight elements most of whose orbits are short). */
 ftk_status ftk_sector_create(ftk_ctx *ctx, const int32_t *perms, int32_t n_g, const double *chi, int32_t n_slots,
                              ftk_sector **out, int64_t *dim_out);
 void ftk_sector_destroy(ftk_sector *sector);

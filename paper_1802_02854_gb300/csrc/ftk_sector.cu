@@ -59,7 +59,7 @@ __device__ __forceinline__ dcx zdiv(dcx a, dcx b) {   // Smith's algorithm
 }
 __device__ __forceinline__ double zabs(dcx a) { return hypot(a.re, a.im); }
 
-constexpr int kMaxGroup = 32;      // group elements (5 bits in loc)
+constexpr int kMaxGroup = 32;      // group elements
 constexpr int kSecThreads = 256;
 constexpr int kScanBlock = 4096;   // states per counting block
 
@@ -153,19 +153,42 @@ __global__ void __launch_bounds__(kSecThreads) sec_compact_kernel(SecGroup G, ui
     }
 }
 
-// loc[x] = sector index * 32 + g of a state whose orbit is in the sector,
-// kLocNone of the others. Groups of at most 16 elements leave bit 4 of g free;
-// it marks the orbits of full size (nearly all), whose sqrt(o) ratio is 1.
+// loc[x] of a state whose orbit is in the sector: its sector index above the
+// element g; kLocNone of the others. Below 2^27 basis vectors the index sits at bit
+// 5, and groups of at most 16 elements leave bit 4 of g free; it marks the orbits
+// of full size (nearly all), whose sqrt(o) ratio is 1. From 2^27 on g takes the bits
+// that the group needs, with the mark above them where there is room (a group whose
+// orbits are nearly all of full size has it: index and element number 2^N states,
+// N <= 30).
 constexpr uint32_t kLocNone = 0xffffffffu;
 constexpr uint32_t kLocFull = 16u;
+constexpr int kLocIndex = 5;
+struct LocBits {
+    int index;                // position of the index
+    uint32_t gmask, full;     // bits of g, mark of a full orbit (0: none)
+};
+// false: dim indices do not fit beside the elements (kLocNone stays free)
+bool loc_bits(int64_t dim, int ng, LocBits *b) {
+    if (dim < 1ll << 27) {
+        *b = {kLocIndex, ng <= (int)kLocFull ? kLocFull - 1 : 31u, ng <= (int)kLocFull ? kLocFull : 0u};
+        return true;
+    }
+    int g = 0;
+    while ((1 << g) < ng) ++g;
+    const int64_t cap = 0xffffffffll >> g;
+    if (dim > cap) return false;
+    const bool mark = dim <= cap >> 1;
+    *b = {g + mark, (1u << g) - 1, mark ? 1u << g : 0u};
+    return true;
+}
 __global__ void sec_loc_kernel(uint64_t dim, const uint32_t *rep_of, const uint8_t *g_of, const int32_t *idx_of,
-                               const int32_t *sec_index, const uint32_t *orb_stab, int flag_full, uint32_t *loc) {
+                               const int32_t *sec_index, const uint32_t *orb_stab, LocBits lb, uint32_t *loc) {
     for (uint64_t x = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; x < dim; x += (uint64_t)gridDim.x * blockDim.x) {
         const int32_t o = idx_of[rep_of[x]], i = sec_index[o];
         uint32_t L = kLocNone;
         if (i >= 0) {
-            L = ((uint32_t)i << 5) | (uint32_t)g_of[x];
-            if (flag_full && orb_stab[o] == 1u) L |= kLocFull;
+            L = ((uint32_t)i << lb.index) | (uint32_t)g_of[x];
+            if (orb_stab[o] == 1u) L |= lb.full;
         }
         loc[x] = L;
     }
@@ -231,7 +254,8 @@ struct SecHvArgs {
     const uint32_t *rep;      // [dim]
     const double *sqo;
     double full;              // sqrt(o) of an orbit of full size
-    int flag_full, ng;        // loc marks them (kLocFull); group elements
+    LocBits lb;
+    int ng;                   // group elements
     const double2 *chi;       // [ng]
     const double2 *in;
     double2 *out;
@@ -320,7 +344,9 @@ __global__ void __launch_bounds__(32) lz_shift_kernel(LzShiftArgs a) {
 // the previous Lanczos iteration, which only the next check waits for.
 constexpr int kSecHvThreads = 128;
 constexpr int kSecChunk = 6;
-template <int EPI>
+// WIDE: the table of 2^27 basis vectors and more; its layout at run time costs 1 %
+// of the 20-site case.
+template <int EPI, bool WIDE>
 __global__ void __launch_bounds__(kSecHvThreads) sec_hv_kernel(const __grid_constant__ SecHam h,
                                                               const __grid_constant__ SecHvArgs a) {
     __shared__ double red[(kSecHvThreads / 32) * 2];
@@ -341,14 +367,16 @@ __global__ void __launch_bounds__(kSecHvThreads) sec_hv_kernel(const __grid_cons
     }
     __syncthreads();
     const int blk = blockIdx.x - nsb, nblk = gridDim.x - nsb;
-    const uint32_t gmask = a.flag_full ? kLocFull - 1u : 31u;
+    const uint32_t gmask = WIDE ? a.lb.gmask : a.lb.full ? kLocFull - 1u : 31u;
+    const uint32_t full_bit = WIDE ? a.lb.full : kLocFull;
+    const int index = WIDE ? a.lb.index : kLocIndex;
     const double sc = a.in_scale ? *a.in_scale : 1.0;
     double d0 = 0, d1 = 0;
     for (int64_t i = (int64_t)blk * blockDim.x + threadIdx.x; i < a.dim; i += (int64_t)nblk * blockDim.x) {
         const uint32_t r = a.rep[i];
         const double so = a.sqo[i];
         const double2 v = a.in[i];
-        const bool full = a.flag_full && so == a.full;
+        const bool full = a.lb.full && so == a.full;
         double ar = 0, ai = 0;
         int anti[3] = {0, 0, 0};
 #pragma unroll
@@ -370,13 +398,13 @@ __global__ void __launch_bounds__(kSecHvThreads) sec_hv_kernel(const __grid_cons
                 anti[g] += __popc(odd);
 #pragma unroll
                 for (int u = 0; u < kSecChunk; ++u)
-                    if (L[u] != kLocNone) w[u] = a.in[L[u] >> 5];
+                    if (L[u] != kLocNone) w[u] = a.in[L[u] >> index];
 #pragma unroll
                 for (int u = 0; u < kSecChunk; ++u)
                     if (L[u] != kLocNone) {
                         double2 t = tab[(2 * g + ((odd >> u) & 1)) * kMaxGroup + (L[u] & gmask)];
-                        if (!full || !(L[u] & kLocFull)) {
-                            const double f = so / a.sqo[L[u] >> 5];
+                        if (!full || !(L[u] & full_bit)) {
+                            const double f = so / a.sqo[L[u] >> index];
                             t.x *= f;
                             t.y *= f;
                         }
@@ -546,6 +574,7 @@ struct ftk_sector {
     // device
     uint32_t *tab = nullptr;             // [ng][nbytes][256]
     uint32_t *loc = nullptr;             // [2^N]
+    LocBits lb{};
     uint32_t *orb_rep = nullptr, *orb_stab = nullptr;   // [n_orb]
     int32_t *sec_index = nullptr;        // [n_orb]
     int32_t *sec_orbit = nullptr;        // [dim]
@@ -615,7 +644,7 @@ SecHvArgs hv_args(ftk_sector *s, const double2 *in, double2 *out) {
     a.rep = s->sec_rep;
     a.sqo = s->sqo;
     a.full = std::sqrt((double)s->ng);
-    a.flag_full = s->ng <= (int)kLocFull;
+    a.lb = s->lb;
     a.ng = s->ng;
     a.chi = s->dchi;
     a.in = in;
@@ -625,6 +654,14 @@ SecHvArgs hv_args(ftk_sector *s, const double2 *in, double2 *out) {
     a.counter = s->counter;
     a.result = s->scal + SC_DOT;
     return a;
+}
+
+template <int EPI>
+void launch_sec_hv(ftk_sector *s, const SecHvArgs &a, int grid) {
+    if (s->dim < 1ll << 27)
+        sec_hv_kernel<EPI, false><<<grid, kSecHvThreads, 0, s->ham.stream>>>(s->sh, a);
+    else
+        sec_hv_kernel<EPI, true><<<grid, kSecHvThreads, 0, s->ham.stream>>>(s->sh, a);
 }
 
 // |v|^2 of a sector vector to *n2 (synchronises)
@@ -805,6 +842,8 @@ ftk_status ftk_sector_create(ftk_ctx *ctx, const int32_t *perms, int32_t n_g, co
     for (long o = 0; o < tot; ++o) { pos[o] = (int)dim; dim += fl[o]; }
     sec->dim = dim;
     if (dim == 0) return fail_all(FTK_EINVAL, "ftk_sector_create: the sector is empty");
+    if (!loc_bits(dim, n_g, &sec->lb))
+        return fail_all(FTK_EINVAL, "ftk_sector_create: more basis vectors than the state table can number");
     CK2(cudaMemcpyAsync(fpos, pos.data(), sizeof(int) * tot, cudaMemcpyHostToDevice, st));
     CK2(cudaMalloc(&sec->sec_index, sizeof(int32_t) * tot));
     CK2(cudaMalloc(&sec->sec_orbit, sizeof(int32_t) * dim));
@@ -814,7 +853,7 @@ ftk_status ftk_sector_create(ftk_ctx *ctx, const int32_t *perms, int32_t n_g, co
                                                                 sec->sec_index, sec->sec_orbit, sec->sec_rep, sec->sqo);
     CK2(cudaGetLastError());
     sec_loc_kernel<<<ggrid, kSecThreads, 0, st>>>(D, rep_of, g_of, idx_of, sec->sec_index, sec->orb_stab,
-                                                  n_g <= (int)kLocFull, sec->loc);
+                                                  sec->lb, sec->loc);
     CK2(cudaGetLastError());
     CK2(cudaMalloc(&sec->vec, sizeof(double2) * (size_t)dim * n_slots));
     CK2(cudaMemsetAsync(sec->vec, 0, sizeof(double2) * (size_t)dim * n_slots, st));
@@ -905,7 +944,7 @@ ftk_status ftk_sector_hv(ftk_sector *sec, int32_t slot_in, int32_t slot_out) {
     if (!sec || slot_in < 0 || slot_out < 0 || slot_in >= sec->n_slots || slot_out >= sec->n_slots || slot_in == slot_out)
         return sfail(sec, FTK_EINVAL, "ftk_sector_hv: bad slots");
     SecHvArgs a = hv_args(sec, slot_ptr(sec, slot_in), slot_ptr(sec, slot_out));
-    sec_hv_kernel<SEC_PLAIN><<<hv_grid(sec), kSecHvThreads, 0, sec->ham.stream>>>(sec->sh, a);
+    launch_sec_hv<SEC_PLAIN>(sec, a, hv_grid(sec));
     SCK(cudaGetLastError());
     ++*sec->ham.launches;
     return FTK_OK;
@@ -958,7 +997,7 @@ ftk_status ftk_sector_tpq(ftk_sector *sec, int32_t slot_state, int32_t slot_work
             a.next_scale = scale + ((k + 1) & 1);
             a.stat_e = stat + (k - k0);
             a.stat_q2 = stat + kStatCap + (k - k0);
-            sec_hv_kernel<SEC_TPQ><<<hv_grid(sec), kSecHvThreads, 0, st>>>(sec->sh, a);
+            launch_sec_hv<SEC_TPQ>(sec, a, hv_grid(sec));
             SCK(cudaGetLastError());
             ++*sec->ham.launches;
         }
@@ -1085,7 +1124,7 @@ ftk_status ftk_sector_green(ftk_sector *sec, int32_t slot, const double *shifts,
             a.done = sec->iflag;
             a.iter = it;
             if (it > 0) a.lz = shift_args(it - 1);
-            sec_hv_kernel<SEC_DOT><<<hv_grid(sec) + a.lz.n_blocks, kSecHvThreads, 0, st>>>(sec->sh, a);
+            launch_sec_hv<SEC_DOT>(sec, a, hv_grid(sec) + a.lz.n_blocks);
             LzArgs u{};
             u.dim = sec->dim;
             u.w = w;
