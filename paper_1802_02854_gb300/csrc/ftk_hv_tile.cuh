@@ -104,11 +104,12 @@ __device__ __forceinline__ unsigned long long odd_bonds(const PassDesc &pd, int 
 // instructions per FP32 pair).
 template <bool ZF>
 struct BondWalk {
-    int q = 0;
+    int q;
     unsigned long long odd;   // shifted along: bit 0 belongs to bond q
     uint32_t classes;
     const PassDesc &pd;
-    __device__ BondWalk(const PassDesc &p, unsigned long long o) : odd(o), classes(p.classes), pd(p) {}
+    __device__ BondWalk(const PassDesc &p, unsigned long long o, int start = 0)
+        : q(start), odd(o >> start), classes(p.classes), pd(p) {}
     template <int TYPE, int SWAP, int KM, class P, class F>
     __device__ __forceinline__ void run(const char *buf, int at, int step, F f) {
         constexpr int c = bond_class(ZF, TYPE, SWAP, KM);
@@ -329,11 +330,17 @@ __device__ __forceinline__ void hv_tile_body(const typename I::amp *__restrict__
         __syncthreads();
         I acc[kTileE];
         const char *cb = reinterpret_cast<const char *>(cur);
+        // z bonds first, with the smaller coefficients; FP64 has them last in its
+        // order, behind y and x
         BondWalk<(I::SH > 0)> bw(pd, odd);
-        if (I::SH > 0) tile_bonds<2>(acc, cb, t * 16, T * 16, bw);
+        if constexpr (I::SH > 0) {
+            tile_bonds<2>(acc, cb, t * 16, T * 16, bw);
+        } else {
+            BondWalk<false> bz(pd, odd, pd.f_end[bond_class(false, 2, 0, 0) - 1]);
+            tile_bonds<2>(acc, cb, t * 16, T * 16, bz);
+        }
         tile_bonds<1>(acc, cb, t * 16, T * 16, bw);
         tile_bonds<0>(acc, cb, t * 16, T * 16, bw);
-        if (I::SH == 0) tile_bonds<2>(acc, cb, t * 16, T * 16, bw);
         // the diagonal last: added first, its size would set the rounding of
         // every term after it
 #pragma unroll

@@ -72,3 +72,13 @@ def test_one_launch_product(prec, n, J):
     cl = named(n)
     v = random_vectors(n, 1, 5)[0]
     assert _error(cl, J, prec, v, 0) <= SLACK[prec] * _expected(cl, J, prec, [(2, 0), (1,)])
+
+
+@pytest.mark.parametrize("n,J", [(12, 0.1), (12, -0.2)])
+def test_floating_point_pass(n, J):
+    """FP64 in one tile, a vector with a neighbourhood of zeros (fixed point takes
+    none): z, y and x bonds in one chain."""
+    cl = named(n)
+    v = random_vectors(n, 1, 5)[0]
+    v[[77] + [77 ^ (1 << i) ^ (1 << j) for i, j, _ in cl.bonds.tolist()]] = 0
+    assert _error(cl, J, "fp64", v, 12) <= SLACK["fp64"] * _expected(cl, J, "fp64", [(2, 1, 0)])
