@@ -23,8 +23,7 @@
  *   and are reduced across threads in double.
  *   FTK_DF is the mixed mode with H.v in double-float arithmetic on the FP32
  *   pipe (hi + lo float pairs in and out, ~48 bits): FP64-class accuracy at
- *   the FP32 pipe's issue rate; its residual update runs inside the first H.v
- *   pass of the next step. The mTPQ state is FP64 in every mode.
+ *   the FP32 pipe's issue rate. The mTPQ state is FP64 in every mode.
  * Memory: device vectors live in ONE caller-allocated device workspace
  *   (ftk_footprint gives its size, ftk_bind_workspace hands it over); the
  *   library never allocates vector-sized memory itself. The context owns only
@@ -405,8 +404,9 @@ ftk_status ftk_plan_info(const ftk_ctx *ctx, int32_t *n_passes, int32_t *tile_bi
 /* Site relabelling that lets H.v run in fewer tiled passes (the layout
  * choice of Sec. IV.A's Hamiltonian-vector product on this hardware: the
  * chunk sites, i.e. the lowest index bits, sit in every tile). Host only, no
- * device work. bonds as in ftk_create; precision and n_rhs select the tile
- * shape (tile_bits 0 = the default). perm_out (host, n_sites ints) receives
+ * device work. bonds as in ftk_create; the precision selects the tile shape
+ * (tile_bits 0 = the default); n_rhs (a power of two <= 32) has no effect, since a
+ * tile holds one vector. perm_out (host, n_sites ints) receives
  * site l -> new label perm_out[l]; relabel the sites (and their positions)
  * before ftk_create. n_passes_out (may be NULL) receives the pass count.
  * The search is deterministic: seeded choices of the chunk sites with greedy

@@ -169,7 +169,7 @@ bool plan_passes(ftk_ctx *ctx, int prec, int tile_bits, Plan &pl, long local_ste
     PlanBond pb[2 * FTK_MAX_PASS_BONDS];
     for (int q = 0; q < ctx->nb; ++q) pb[q] = {ctx->bonds[q].i, ctx->bonds[q].j, ctx->bonds[q].g};
     PassDesc pd[FTK_MAX_PASSES];
-    const int np = plan_hv_passes(ctx->n, pb, ctx->nb, ctx->K, ctx->J, elem_bytes(prec), 1, tile_bits, pd,
+    const int np = plan_hv_passes(ctx->n, pb, ctx->nb, ctx->K, ctx->J, elem_bytes(prec), tile_bits, pd,
                                   FTK_MAX_PASSES, &pl.tile_bits, &pl.chunk_bits, 32, local_steps);
     if (np == 0) return false;
     if (hv_tiled(prec, pd[0])) {
@@ -905,7 +905,7 @@ static ftk_status cocg_core(ftk_ctx *ctx, const CocgReq &rq, double *G_out, int3
     LAUNCH(launch_cocg_update(upd_kind(ctx), B, nullptr, nullptr, rcur, ua, upd_grid(ctx, B), ctx->stream));
     int it0 = 0;
     if (ctx->prec == FTK_DF) {
-        // step 0 without the fused update: W = H r_0 (+mu), seed, shifts
+        // step 0 has no update before it: W = H r_0 (+mu), seed, shifts
         EpiArgs e0 = ea;
         e0.df_lo = ua.lo_stride;
         if ((s = run_hv(ctx, ctx->mprec, B, EPI_COCG, rcur, w, e0))) return s;
@@ -1612,7 +1612,7 @@ ftk_status ftk_suggest_order(int32_t n_sites, const ftk_bond *bonds, int32_t n_b
     int tb = tile_bits > 0 ? std::min((int)tile_bits, tb_max) : tb_max;
     tb = std::max(2, std::min(tb, (int)n_sites));
     int perm[FTK_MAX_SITES];
-    const int np = plan_suggest_order(n_sites, pb, n_bonds, elem_bytes(prec), 1, tb, perm);
+    const int np = plan_suggest_order(n_sites, pb, n_bonds, elem_bytes(prec), tb, perm);
     if (np == 0) return fail(nullptr, FTK_EINVAL, "ftk_suggest_order: planning failed");
     for (int s = 0; s < n_sites; ++s) perm_out[s] = perm[s];
     if (n_passes_out) *n_passes_out = np;

@@ -55,7 +55,7 @@ __device__ __forceinline__ void bond_apply_df(float2 (&ah)[1 << LE], float2 (&al
 
 #define FTK_HV_DF_CASE(ID, KA, KB)                                                                   \
     case ID:                                                                                         \
-        if constexpr (KA < LE && KB < LE) bond_apply_df<LE, KA, KB>(ah, al, ph, pl, cf);             \
+        bond_apply_df<LE, KA, KB>(ah, al, ph, pl, cf);                                               \
         break;
 
 // TB > 0: the thread bits of the tile (tile_bits - LE) as a compile-time
@@ -83,7 +83,7 @@ hv_df_kernel(const float2 *__restrict__ in, float2 *out, long long ld, const __g
     uint64_t st = 0;
     for (int q = 0; q < tb; ++q)
         if ((t >> q) & 1) st |= 1ull << pd.tile_pos[q];
-    long long kofs[LE > 0 ? LE : 1];
+    long long kofs[LE];
 #pragma unroll
     for (int q = 0; q < LE; ++q) kofs[q] = (long long)(1ull << pd.tile_pos[tb + q]);
     auto eofs = [&](int k) -> long long {
@@ -116,8 +116,9 @@ hv_df_kernel(const float2 *__restrict__ in, float2 *out, long long ld, const __g
         const uint64_t m = free_mask;
         return (long long)((((uint64_t)ofs | ~m) + dep_grid) & m);
     };
-    // diagonal dgv[0] c0 + dgv[1] c1 (integer counts c as in the kernel
-    // above) in double-float arithmetic, once per thread
+    // diagonal dgv[0] c0 + dgv[1] c1 in double-float arithmetic, once per thread: c
+    // counts the parallel minus the antiparallel bonds, c0 of the x and y bonds, c1 of
+    // the z bonds
     float dgh[E], dgl[E];
     {
         int c0[E], c1[E];
@@ -206,13 +207,9 @@ hv_df_kernel(const float2 *__restrict__ in, float2 *out, long long ld, const __g
                         FTK_HV_DF_CASE(1, 0, -1)
                         FTK_HV_DF_CASE(2, 1, -1)
                         FTK_HV_DF_CASE(3, 2, -1)
-                        FTK_HV_DF_CASE(4, 3, -1)
                         FTK_HV_DF_CASE(9 + 0 * 8 + 1, 0, 1)
                         FTK_HV_DF_CASE(9 + 0 * 8 + 2, 0, 2)
-                        FTK_HV_DF_CASE(9 + 0 * 8 + 3, 0, 3)
                         FTK_HV_DF_CASE(9 + 1 * 8 + 2, 1, 2)
-                        FTK_HV_DF_CASE(9 + 1 * 8 + 3, 1, 3)
-                        FTK_HV_DF_CASE(9 + 2 * 8 + 3, 2, 3)
                         default: break;
                     }
                 }

@@ -109,7 +109,7 @@ struct BondWalk {
     uint32_t classes;
     const PassDesc &pd;
     __device__ BondWalk(const PassDesc &p, unsigned long long o, int start = 0)
-        : q(start), odd(o >> start), classes(p.classes), pd(p) {}
+        : q(start), odd(start < 64 ? o >> start : 0), classes(p.classes), pd(p) {}
     template <int TYPE, int SWAP, int KM, class P, class F>
     __device__ __forceinline__ void run(const char *buf, int at, int step, F f) {
         constexpr int c = bond_class(ZF, TYPE, SWAP, KM);

@@ -101,7 +101,7 @@ extern "C" ftk_status ftk_tpq_step_noalloc(int32_t n_sites, const ftk_bond *bond
     const bool gather = hv_use_gather(0, n_sites, 1) && gather_desc(n_sites, pb, n_bonds, K, J, &gd);
     PassDesc pd[FTK_MAX_PASSES];
     int tb = 0, cb = 0;
-    const int np = gather ? 0 : plan_hv_passes(n_sites, pb, n_bonds, K, J, 16, 1, hv_max_tile_bits(0), pd, FTK_MAX_PASSES,
+    const int np = gather ? 0 : plan_hv_passes(n_sites, pb, n_bonds, K, J, 16, hv_max_tile_bits(0), pd, FTK_MAX_PASSES,
                                   &tb, &cb);
     if (np == 0 && !gather) return noalloc_fail(FTK_EINVAL, "ftk_tpq_step_noalloc: pass planning failed");
     for (int p = 0; p < np; ++p)

@@ -231,11 +231,11 @@ constexpr long kPlanLocalSteps = 30000;
 // local_steps > 0: after the greedy covers, a local search (plan_anneal_cover,
 // 8 seeded restarts of local_steps moves) looks for covers with fewer passes.
 inline int plan_hv_passes(int n, const PlanBond *bonds, int nb, double K, double J, int elem_bytes,
-                          int B, int tile_bits, PassDesc *pd, int max_passes, int *b_out, int *c_out,
+                          int tile_bits, PassDesc *pd, int max_passes, int *b_out, int *c_out,
                           int restarts = 32, long local_steps = 0) {
     if (n < 2 || n > FTK_MAX_SITES || nb < 1 || nb > 2 * FTK_MAX_PASS_BONDS) return 0;
     int c = 0;
-    while (c < n && ((long)1 << c) * B * elem_bytes < 256) ++c;
+    while (c < n && ((long)1 << c) * elem_bytes < 256) ++c;
     int b = tile_bits < n ? tile_bits : n;
     if (b < n && c > b - 2) c = b - 2 > 0 ? b - 2 : 0;   // later passes need >= 2 free tile bits
     if (c > b) c = b;
@@ -323,12 +323,12 @@ inline int plan_hv_passes(int n, const PlanBond *bonds, int nb, double K, double
 // (and the given labelling) and returns in perm (site l -> new label
 // perm[l]) the labelling whose plan has the fewest passes; returns that
 // number of passes (0 on failure).
-inline int plan_suggest_order(int n, const PlanBond *bonds, int nb, int elem_bytes, int B, int tile_bits, int *perm,
+inline int plan_suggest_order(int n, const PlanBond *bonds, int nb, int elem_bytes, int tile_bits, int *perm,
                               int trials = 64) {
     PassDesc pd[FTK_MAX_PASSES];
     int b = 0, c = 0;
     for (int s = 0; s < n; ++s) perm[s] = s;
-    int best = plan_hv_passes(n, bonds, nb, -1.0, 0.1, elem_bytes, B, tile_bits, pd, FTK_MAX_PASSES, &b, &c, 16);
+    int best = plan_hv_passes(n, bonds, nb, -1.0, 0.1, elem_bytes, tile_bits, pd, FTK_MAX_PASSES, &b, &c, 16);
     if (best == 0) return 0;
     PlanRng rng{0x9e3779b9u};
     for (int t = 0; t < trials && best > 1; ++t) {
@@ -346,7 +346,7 @@ inline int plan_suggest_order(int n, const PlanBond *bonds, int nb, int elem_byt
             if (!used[s]) cand[s] = next++;
         PlanBond rb[2 * FTK_MAX_PASS_BONDS];
         for (int q = 0; q < nb; ++q) rb[q] = {cand[bonds[q].i], cand[bonds[q].j], bonds[q].g};
-        const int np = plan_hv_passes(n, rb, nb, -1.0, 0.1, elem_bytes, B, tile_bits, pd, FTK_MAX_PASSES, &b, &c, 16);
+        const int np = plan_hv_passes(n, rb, nb, -1.0, 0.1, elem_bytes, tile_bits, pd, FTK_MAX_PASSES, &b, &c, 16);
         if (np > 0 && np < best) {
             best = np;
             for (int s = 0; s < n; ++s) perm[s] = cand[s];
@@ -371,7 +371,7 @@ inline int plan_suggest_order(int n, const PlanBond *bonds, int nb, int elem_byt
                 if (!is_chunk[s]) cand[s] = next++;
             PlanBond rb[2 * FTK_MAX_PASS_BONDS];
             for (int q = 0; q < nb; ++q) rb[q] = {cand[bonds[q].i], cand[bonds[q].j], bonds[q].g};
-            const int np = plan_hv_passes(n, rb, nb, -1.0, 0.1, elem_bytes, B, tile_bits, pd, FTK_MAX_PASSES, &b, &c,
+            const int np = plan_hv_passes(n, rb, nb, -1.0, 0.1, elem_bytes, tile_bits, pd, FTK_MAX_PASSES, &b, &c,
                                           16, kPlanLocalSteps);
             if (np > 0 && np <= target) {
                 best = np;
