@@ -196,7 +196,7 @@ ftk_status get_plan(ftk_ctx *ctx, int prec, int B, Plan **out) {
     auto it = ctx->plans.find(prec * 64 + B);
     if (it != ctx->plans.end()) { *out = &it->second; return FTK_OK; }
     Plan pl;
-    if (ctx->tile_bits_req <= 0 && hv_use_gather(prec, ctx->n, B)) {
+    if (ctx->tile_bits_req <= 0 && hv_use_gather(prec, ctx->n, B, fix_couplings(ctx->K, ctx->J))) {
         pl = whole_gather(ctx);
     } else {   // default: the largest tile
         const int tb_max = hv_max_tile_bits(prec);
@@ -205,9 +205,11 @@ ftk_status get_plan(ftk_ctx *ctx, int prec, int B, Plan **out) {
         if (!plan_passes(ctx, prec, tb, pl))
             return fail(ctx, FTK_EINVAL, "H.v pass planning failed (tile too small for the bond list)");
         // Few tiles per SM: tiles of half the size, two CTAs to an SM, if a
-        // greedy plan finds as few passes for them (20 sites, two FP32 vectors:
-        // 44 -> 35 us). With many tiles one CTA's copies run behind its own
-        // sums, and half tiles mean more passes.
+        // greedy plan finds as few passes for them (FP32, 20 sites, 1, 2 and 4
+        // vectors: 31 -> 26, 44 -> 35, 69 -> 58 us). With many tiles one CTA's
+        // copies run behind its own sums, and half tiles mean more passes (with one
+        // pass more: FP64, 20 sites 69 -> 78 us; FP32, 18 sites 14 -> 16, 24 sites
+        // 218 -> 257).
         if (prec != 2 && ctx->tile_bits_req <= 0 && ctx->n > tb && (B << (ctx->n - tb)) < 4 * ctx->n_sm) {
             Plan half;
             if (plan_passes(ctx, prec, tb - 1, half, 0) && half.n_passes() <= pl.n_passes()) pl = half;
@@ -1582,7 +1584,7 @@ ftk_status ftk_autotune(ftk_ctx *ctx, int32_t n_rhs, int32_t which, int32_t *til
         Plan pl;
         if (plan_passes(ctx, prec, tb, pl)) time_plan(pl);
     }
-    if (st == FTK_OK && hv_use_gather(prec, ctx->n, n_rhs)) time_plan(whole_gather(ctx));
+    if (st == FTK_OK && hv_use_gather(prec, ctx->n, n_rhs, fix_couplings(ctx->K, ctx->J))) time_plan(whole_gather(ctx));
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (st != FTK_OK) return fail(ctx, st, "ftk_autotune: CUDA error while timing");

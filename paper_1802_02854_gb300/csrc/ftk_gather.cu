@@ -218,26 +218,29 @@ void gather_pass(const PassDesc &pd, GatherDesc *gd) {
     *gd = d;
 }
 
-// Where the line lies, us per product of B vectors, gather against the tiled
-// passes (K = -1, J = 0.1):
-//   FP64  18 sites 29 / 37, 20 sites 117 / 66; four vectors: 16 sites 27 / -,
-//         18 sites 107 / 64, 20 sites 461 / 192
-//   FP32  12 sites 3.3 / 11, 18: 11 / 15, 20: 38 / 31; four vectors: 16 sites
-//         10 / -, 18 sites 36 / 23, 20 sites 143 / -
-//   DF    12: 3.7 / 17, 16: 5.8 / 25, 18: 15 / 28, 20: 53 / 65; four vectors
-//         3.7 / 67, 14 / 99, 49 / 110, 201 / 187
-// (-: not measured). FP64 and FP32 cross between 2^18 and 2^19 amplitudes in
-// all, where the gather's L2 reads (and, in FP64, its multiply-adds at the FP64
-// pipe's rate) cost more than the passes' launches and empty SMs; the
-// double-float passes are dearer and cross above 2^20.
-bool hv_use_gather(int prec, int n, int B) {
+// Where the line lies, us per product of B vectors (n sites x B), gather against
+// the tiled passes in their better tile size (K = -1, J = 0.1; products queued one
+// after the other):
+//   all B 2^n      2^17          2^18                      2^19                      2^20
+//   FP64      16x2: 18 / 30   16x4: 31 / 33, 18x1: 34 / 41   16x8: 57 / 37, 18x2: 62 / 43  18x4: 119 / 65
+//   FP32      16x2:  8 /  9   16x4: 12 / 10, 18x1: 13 / 14   16x8: 21 / 13, 18x2: 21 / 14  18x4: 37 / 23
+//   DF        16x2: 10 / 21   16x4: 16 / 21, 18x1: 17 / 28   16x8: 27 / 26, 18x2: 29 / 34  16x16: 49 / 41,
+//                                                                   18x4: 51 / 54, 20x1: 56 / 57
+//             2^21: 18x8: 99 / 94, 20x2: 105 / 96
+// FP64 and FP32 cross at 2^18, where the gather's L2 reads (and, in FP64, its
+// multiply-adds at the FP64 pipe's rate) cost more than the passes' launches and
+// empty SMs; double-float passes are dearer and cross at 2^20. Couplings without a
+// fixed-point form (fix_couplings) leave the FP64 passes to the same pipe, which
+// they use no better: 18x2 62 / 97, 20x1 129 / 178, 20x2 255 / 306, 20x4 505 / 545.
+bool hv_use_gather(int prec, int n, int B, bool fix) {
     int w = n;
     for (int b = 1; b < B; b <<= 1) ++w;
-    return w <= (prec == 2 ? 20 : 18);
+    return w <= (prec == 2 ? 20 : prec == 0 && !fix ? 22 : 18);
 }
 
 // Threads per block: few for the smallest vectors, so that their blocks reach
-// more SMs. Blocks per column: one amplitude per thread, at most 1024 blocks
+// more SMs (32 / 64 / 128 threads, FP64: 14 sites 8.1 / 7.3 / 7.3 us, 16 sites 10.5 /
+// 10.4 / 12.4, 18 sites 33.1 / 34.7 / 34.0; the launch's own time hides it below). Blocks per column: one amplitude per thread, at most 1024 blocks
 // where their partial dots are summed by the last one.
 static int gather_threads(int n) { return n <= 12 ? 32 : n <= 14 ? 64 : 128; }
 

@@ -15,9 +15,9 @@
 // register bits). The group with mask 0 holds the bonds between register sites,
 // and the diagonal.
 //
-// What bounds it: the FP32 pipe, 10 packed f32x2 instructions a term (24 sites,
-// one vector: 684 us, 18 T operations/s of the pipe's 40; 752 us with 12, 775
-// without chained launches). The layout of ftk_hv_tile.cuh (1024 threads, a
+// What bounds it: the latency of 10 dependent packed f32x2 instructions a term at 16
+// warps an SM (24 sites, one vector: 684 us; FMA pipe 51-55 % busy, issue slots
+// 50-54 %; 752 us with 12 instructions, 775 without chained launches). The layout of ftk_hv_tile.cuh (1024 threads, a
 // partner read per bond) ran 812 us against 752: its gain in latency
 // does not outweigh the extra instructions here. Exact float pieces (the sums of
 // ftk_hv_fix.cu on three aligned floats, 4.3 packed instructions a term) ran 959

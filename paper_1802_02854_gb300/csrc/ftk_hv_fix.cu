@@ -436,6 +436,16 @@ static bool range_plan(int n, const PlanBond *bonds, int nb, RangePlan *rp) {
     return total > 0;
 }
 
+// Exponents stay inside the range; and the measured sums count x and y bonds, so
+// both of their coefficients must differ from zero, else some state has no such
+// term and no vector is admitted.
+bool fix_couplings(double K, double J) {
+    const double cmax = std::max(fabs(K), fabs(J)) / 4;
+    double par, anti;
+    bond_coefficients(0, K, J, &par, &anti);
+    return cmax > 0x1p-40 && cmax < 0x1p40 && par != 0 && anti != 0;
+}
+
 // Coefficients and scales for the passes of one plan, and its measuring launch.
 // Sums: a pass of nb bonds adds at most nb amplitudes to A and 3 nb to B (the
 // antiparallel ones twice, and the diagonal), which has to stay below 2^63 with
@@ -445,8 +455,7 @@ static bool range_plan(int n, const PlanBond *bonds, int nb, RangePlan *rp) {
 // Admission, with q the input's quantum: an output's error is at most q / 2 for each
 // unit of its coefficients (at most bound in all), and per pass the roundings of
 // fix_combine. need is where that equals (nb + 1) 2^-53 of the sum of its terms'
-// sizes. The sum counts x and y bonds, so both of their coefficients must differ
-// from zero, else some state has no such term and no vector is admitted.
+// sizes.
 bool fix_plan(PassDesc *pd, int np, const PlanBond *bonds, int nb, double K, double J, RangePlan *rp) {
     int most = 1;
     for (int p = 0; p < np; ++p) {
@@ -454,11 +463,10 @@ bool fix_plan(PassDesc *pd, int np, const PlanBond *bonds, int nb, double K, dou
         if (!hv_tiled(0, pd[p]) || pd[p].n_bonds > 60) return false;
         most = std::max(most, pd[p].n_bonds);
     }
+    if (!fix_couplings(K, J) || !range_plan(pd[0].n_sites, bonds, nb, rp)) return false;
     const double cmax = std::max(fabs(K), fabs(J)) / 4;
-    if (!(cmax > 0x1p-40) || !(cmax < 0x1p40)) return false;   // exponents stay inside the range
     double par, anti;
     bond_coefficients(0, K, J, &par, &anti);
-    if (par == 0 || anti == 0 || !range_plan(pd[0].n_sites, bonds, nb, rp)) return false;
     int ec = 0;
     if (frexp(cmax, &ec) == 0.5) --ec;   // cmax <= 2^ec
     double bound = 0;

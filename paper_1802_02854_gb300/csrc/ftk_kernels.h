@@ -244,7 +244,7 @@ bool hv_tiled(int prec, const PassDesc &pd);
 struct PlanBond;
 bool gather_desc(int n, const PlanBond *bonds, int nb, double K, double J, GatherDesc *gd);
 void gather_pass(const PassDesc &pd, GatherDesc *gd);   // the bonds of a planned pass
-bool hv_use_gather(int prec, int n, int B);
+bool hv_use_gather(int prec, int n, int B, bool fix);
 cudaError_t launch_hv_gather(int prec, int B, int epi, const void *in, void *out, const GatherDesc &gd,
                              const EpiArgs &ea, cudaStream_t st);
 // FP64 passes in fixed point (ftk_hv_fix.cu): coefficients of a laid-out plan
@@ -252,6 +252,7 @@ cudaError_t launch_hv_gather(int prec, int B, int epi, const void *in, void *out
 // for B vectors: range has to be zero, other (may be NULL) is cleared for the next
 // launch, once the products that read it are through.
 bool fix_plan(PassDesc *pd, int np, const PlanBond *bonds, int nb, double K, double J, RangePlan *rp);
+bool fix_couplings(double K, double J);   // false: no plan of such couplings has
 cudaError_t fix_attributes();
 cudaError_t launch_fix_range(const void *in, int n, int B, FixRange *range, FixRange *other, const RangePlan &rp,
                              const EpiArgs &ea, int n_sm, cudaStream_t st);

@@ -98,7 +98,7 @@ extern "C" ftk_status ftk_tpq_step_noalloc(int32_t n_sites, const ftk_bond *bond
 
     // plan (stack only): FP64, one vector; the product of a small one is one launch
     GatherDesc gd;
-    const bool gather = hv_use_gather(0, n_sites, 1) && gather_desc(n_sites, pb, n_bonds, K, J, &gd);
+    const bool gather = hv_use_gather(0, n_sites, 1, fix_couplings(K, J)) && gather_desc(n_sites, pb, n_bonds, K, J, &gd);
     PassDesc pd[FTK_MAX_PASSES];
     int tb = 0, cb = 0;
     const int np = gather ? 0 : plan_hv_passes(n_sites, pb, n_bonds, K, J, 16, hv_max_tile_bits(0), pd, FTK_MAX_PASSES,

@@ -197,3 +197,36 @@ def test_iteration_and_solve(ftk, kind):
         ctx.close()
     for g in G[1:]:
         assert np.abs(g - G[0]).max() <= 1e-9 * np.abs(G[0]).max()
+
+
+@pytest.mark.parametrize("n,B", [(18, 2), (20, 1), (20, 4)])
+@pytest.mark.parametrize("K,J", [(0.0, 1.0), (0.4, -0.2)])
+def test_couplings_without_fixed_point(ftk, K, J, n, B):
+    """An x or y coefficient of zero: one launch up to 2^22 amplitudes, through
+    the block product, the iteration and the step on the caller's buffers; norm
+    error within that of a chain over all terms."""
+    import torch
+    cl = named(n)
+    vs = random_vectors(n, B, 12)
+    ctx = ftk.Context(cl, K, J, "fp64", max_rhs=B, n_saved=1)
+    assert ctx.plan_info() == (1, n)
+    out = ctx.hv(torch.from_numpy(vs if B > 1 else vs[0]).cuda())
+    torch.cuda.synchronize()
+    got = out.cpu().numpy().reshape(vs.shape)
+    ref = [sparse.hv(cl, K, J, v) for v in vs]
+    bound = (len(cl.bonds) + 4) * 2.0 ** -53 * 2 * len(cl.bonds) * max(abs(K), abs(J))
+    for v, g, r in zip(vs, got, ref):
+        assert np.linalg.norm(g - r) <= bound * np.linalg.norm(v)
+    psi = vs[0] / np.linalg.norm(vs[0])
+    ell = 2.0
+    ctx.set_state(psi, ell)
+    u, _, h2 = ctx.tpq_step(2, 100)
+    ctx.close()
+    w = sparse.hv(cl, K, J, psi)
+    assert abs(u[0] - np.vdot(psi, w).real / n) < 1e-12
+    p = torch.from_numpy(psi).cuda()
+    o = torch.empty_like(p)
+    stats = ftk.ftk_tpq_step_noalloc(n, cl.bonds, K, J, ell, p.data_ptr(), o.data_ptr(),
+                                     torch.cuda.current_stream().cuda_stream)
+    assert abs(stats[0] - u[0]) < 1e-12 and abs(stats[1] - h2[0]) < 1e-9 * abs(h2[0])
+    assert np.linalg.norm(o.cpu().numpy() - (ell * psi - w / n)) <= 1e-13
