@@ -25,7 +25,7 @@
 // fix_range_kernel measures before each product, for every output and for real and
 // imaginary parts apart, a lower bound of the sum of its terms' sizes, and a vector
 // is admitted where the fixed-point error bound stays at every output within that
-// of the chain, (bonds + 1) 2^-53 of the sum (fix_plan). Any other vector (zeros or
+// of the chain, (bonds + 4) 2^-53 of the sum (fix_plan). Any other vector (zeros or
 // tiny blocks, very wide ranges, extreme exponents, infinities, NaN) takes the
 // floating-point pass (hv_tile_body), inside the same launches. (Admission by the
 // mean distance of the exponents from the largest let blocks of tiny components
@@ -63,8 +63,8 @@ namespace ftk {
 
 // ---------------------------------------------------------------- measuring
 // Largest exponent of a vector's components and the smallest of its outputs'
-// sums of term sizes, over the x and y bonds inside tiles of 2^14 amplitudes (12
-// to 14 bonds on the honeycomb clusters; a term left out only lowers the bound).
+// sums of term sizes, over the x and y bonds inside tiles of 2^13 or 2^14 amplitudes
+// (12 to 14 bonds on the honeycomb clusters; a term left out only lowers the bound).
 // Grid (split x persistent CTAs, columns): the outputs of a tile are shared by
 // split CTAs that all load it. A tile is held as bf16 sizes (rounded down, so that
 // the sums stay lower bounds; FixCoef::need holds the additions' rounding), four
@@ -394,11 +394,10 @@ hv_fix_kernel(const double2 *__restrict__ in, double2 *out, long long ld, const 
 // ===================================================================== host
 // The measuring launch's tile: the lowest sites (contiguous runs of 128 bytes),
 // and greedily the sites with the most x and y bonds into it; its bonds, by which
-// of the sites 0 and 1 (the bits inside an item) they flip. Returns false if it
-// holds none.
-static bool range_plan(int n, const PlanBond *bonds, int nb, RangePlan *rp) {
+// of the sites 0 and 1 (the bits inside an item) they flip. Returns their number.
+static int range_plan(int n, const PlanBond *bonds, int nb, int bits, RangePlan *rp) {
     RangePlan r{};
-    r.bits = std::min(n, kRangeBits);
+    r.bits = std::min(n, bits);
     r.n_free = n - r.bits;
     int at[FTK_MAX_SITES];   // offset bit of a site, -1: not in the tile
     std::fill(at, at + FTK_MAX_SITES, -1);
@@ -433,7 +432,7 @@ static bool range_plan(int n, const PlanBond *bonds, int nb, RangePlan *rp) {
         ++total;
     }
     *rp = r;
-    return total > 0;
+    return total;
 }
 
 // Exponents stay inside the range; and the measured sums count x and y bonds, so
@@ -454,8 +453,10 @@ bool fix_couplings(double K, double J) {
 // product (at most sum_b (|off-diagonal| + |diagonal|) max |v|) below 2^62.
 // Admission, with q the input's quantum: an output's error is at most q / 2 for each
 // unit of its coefficients (at most bound in all), and per pass the roundings of
-// fix_combine. need is where that equals (nb + 1) 2^-53 of the sum of its terms'
-// sizes.
+// fix_combine. need is where that equals (nb + 3) 2^-53 of the sum of its terms'
+// sizes; the result's rounding makes it nb + 4, what a chain of multiply-adds may
+// lose: one for each bond, the diagonal and the partial product, two for the
+// diagonal's coefficient.
 bool fix_plan(PassDesc *pd, int np, const PlanBond *bonds, int nb, double K, double J, RangePlan *rp) {
     int most = 1;
     for (int p = 0; p < np; ++p) {
@@ -463,7 +464,13 @@ bool fix_plan(PassDesc *pd, int np, const PlanBond *bonds, int nb, double K, dou
         if (!hv_tiled(0, pd[p]) || pd[p].n_bonds > 60) return false;
         most = std::max(most, pd[p].n_bonds);
     }
-    if (!fix_couplings(K, J) || !range_plan(pd[0].n_sites, bonds, nb, rp)) return false;
+    if (!fix_couplings(K, J)) return false;
+    // tiles of 2^13 if they hold 12 bonds (18 sites, one and four vectors 6.7 and 8.4 us
+    // for 8.7 and 11.0; random vectors of up to 2^27 components pass with 12), else of
+    // 2^14 (20 sites: 12 bonds for 11)
+    if (range_plan(pd[0].n_sites, bonds, nb, kRangeBits - 1, rp) < 12 &&
+        range_plan(pd[0].n_sites, bonds, nb, kRangeBits, rp) == 0)
+        return false;
     const double cmax = std::max(fabs(K), fabs(J)) / 4;
     double par, anti;
     bond_coefficients(0, K, J, &par, &anti);
@@ -487,17 +494,18 @@ bool fix_plan(PassDesc *pd, int np, const PlanBond *bonds, int nb, double K, dou
     f.jl = (int)(ji & ((1 << 30) - 1));
     f.ex = 1 - 1023 - (53 + f.lsh) + ec + 2 + f.sr;
     // the coefficients' bf16 sizes, rounded down
-    const float cp = (float)fabs(par), ca = (float)fabs(anti);
-    auto below = [](float x) -> uint32_t {   // also where x itself was rounded up
+    auto below = [](double c) -> uint32_t {
+        const float x = (float)c;
         uint32_t u;
         memcpy(&u, &x, 4);
-        u = (u >> 16) > 0 ? (u >> 16) - 1 : 0;
+        if ((double)x > c && (u & 0xffffu) == 0) --u;   // rounded up to a bf16 number
+        u >>= 16;
         return u << 16 | u;
     };
-    rp->par = below(cp);
-    rp->anti = below(ca);
+    rp->par = below(fabs(par));
+    rp->anti = below(fabs(anti));
     const double combine = 1 + ((double)f.kl + f.jl) * 0x1p-31 + (f.sr > 0);
-    const double need = (bound / 2 + np * combine * ldexp(1.0, ec + 2 + f.sr)) / (ldexp(1.0, f.lsh) * (nb + 1));
+    const double need = (bound / 2 + np * combine * ldexp(1.0, ec + 2 + f.sr)) / (ldexp(1.0, f.lsh) * (nb + 3));
     f.need = (float)(need * pow(1 + 0x1p-8, rp->n[0] + rp->n[1] + rp->n[2] + rp->n[3] + 2));   // bf16 additions, the float product
     for (int p = 0; p < np; ++p) pd[p].fx = f;
     return true;
