@@ -76,7 +76,7 @@ FP64_PEAK_TFLOPS = 1.25
 # dram__bytes_read.sum + dram__bytes_write.sum summed over the three passes of
 # the 24-site plan with 2^12-amplitude tiles (one column, --hv-only); valid
 # for that plan of the current kernel only
-DF_HV_DRAM_BYTES = 1996.7e6     # 1342.4 MB read + 654.3 MB written
+DF_HV_DRAM_BYTES = 1996.2e6     # 1342.5 MB read + 653.7 MB written
 DF_HV_DRAM_PLAN = (24, 3, 12)    # (sites, passes, tile bits) the counters were taken on
 
 

@@ -32,14 +32,14 @@
 // come out as 0.)
 //
 // Measured, relative to the norm of the product, against double-double sums, random
-// vectors, typical states and residuals at 18 to 24 sites: 6.0e-17 to 1.2e-16; the
-// chain of multiply-adds 8.6e-17 to 1.4e-16. At the worst component of any of them 3.8
+// vectors, typical states and residuals at 18 to 24 sites: 6.0e-17 to 1.3e-16; the
+// chain of multiply-adds 8.6e-17 to 1.4e-16. At the worst component of any of them 3.1
 // 2^-53 of its terms; the chain 3.4, admission by the mean exponent 7.9.
 //
 // What bounds it now: the issue slots and the integer pipe (24 sites, three
 // passes: 208, 226 and 246 us, 61-68 % of the issue slots and 48-55 % of the ALU;
-// with the measuring launch 751 us per product for 2412; a vector that is not
-// admitted 2365; 18 sites, four vectors: 70 for 166, not admitted 175).
+// with the measuring launch 753 us per product for 2412; a vector that is not
+// admitted 2362; 18 sites, four vectors: 68 for 166, not admitted 173).
 //
 // Layout and items as in ftk_hv_tile.cuh (1024 threads of 4 amplitudes: 32 warps
 // hide the latencies that 16 warps of 8 or 8 of 16 did not). The y bonds come
@@ -70,7 +70,7 @@ namespace ftk {
 // the sums stay lower bounds; FixCoef::need holds the additions' rounding), four
 // neighbouring amplitudes in 16 bytes. Sizes below the float range count as 0,
 // which refuses.
-// What bounds it: at 24 sites the read (50 us of 74) and, after it, the shared reads
+// What bounds it: at 24 sites the read (50 us of 75) and, after it, the shared reads
 // of 4 bytes a bond and amplitude (128 bytes a cycle and SM); below 20 sites one
 // tile's time, which split shortens.
 constexpr int kRangeThreads = 1024, kRangeCtas = 2, kRangeE = (1 << (kRangeBits - 2)) / kRangeThreads;   // items a thread
