@@ -101,7 +101,9 @@ struct ftk_ctx {
     GatherDesc gd{};
     // The next product measures into range[range_slot], which the launch before
     // cleared. A captured solve holds an even number of products, so that the turns
-    // go on after any number of its launches.
+    // go on after any number of its launches. (What a caller's own capture of an odd
+    // number would leave in a slot, larger exponents and smaller sums, can only
+    // refuse a vector.)
     int range_slot = 0;
     std::vector<double> pos;
     cudaStream_t stream = nullptr;

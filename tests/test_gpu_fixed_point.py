@@ -151,6 +151,29 @@ def test_measured_afresh(ftk):
     ctx.close()
 
 
+def test_captured_product(ftk):
+    """A single product in a caller's graph, replayed on changing inputs."""
+    import torch
+    cl = named(N)
+    ctx = ftk.Context(cl, -1.0, 0.1, "fp64", tile_bits=12)
+    v = torch.zeros(1 << N, dtype=torch.complex128, device="cuda")
+    out = torch.empty_like(v)
+    graph = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph, stream=ctx.stream):
+        ftk.ftk_hv(ctx.handle, v.data_ptr(), out.data_ptr(), 1)
+    for kind, scale in (("gauss", 1.0), ("typical", 2.0 ** 30), ("edge-70", 1.0), ("gauss", 2.0 ** -40), ("gauss", 1.0)):
+        x = scale * _vector(cl, kind)
+        v.copy_(torch.from_numpy(x))
+        graph.replay()
+        torch.cuda.synchronize()
+        _check(cl, -1.0, 0.1, x, out.cpu().numpy())
+        direct = ctx.hv(v)
+        torch.cuda.synchronize()
+        _check(cl, -1.0, 0.1, x, direct.cpu().numpy())
+    ctx.close()
+
+
 def test_denormal_components(ftk):
     """Products of the smallest numbers are rounded, not dropped: within one
     quantum per term, and a half for each multiple that is formed."""
